@@ -274,7 +274,8 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         e = launch_cull(cv, vt, base, slot->scratch, st);
         if (e != cudaSuccess) return cuda_fail(e, "cull launch");
         if (fe) cudaEventRecord(fe->ev[2], st);
-        e = launch_raster(cv, vt, base, slot->scratch, shape, st);
+        int raster_kernels = 0;
+        e = launch_raster(cv, vt, base, slot->scratch, shape, st, &raster_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "raster launch");
         if (fe) cudaEventRecord(fe->ev[3], st);
         if (shade) {
@@ -287,7 +288,7 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         e = launch_resolve(cv, vt, slot->scratch, st);
         if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
         if (fe) cudaEventRecord(fe->ev[5], st);
-        launches += 4;
+        launches += 3 + raster_kernels;
         raster_launches += 1;
     }
     return PC_OK;

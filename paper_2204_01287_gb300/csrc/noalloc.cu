@@ -135,7 +135,9 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     shape.blocks = 0;   // one resident wave
     if (launch_clear(vt, 0, s, st) != cudaSuccess) return PC_ECUDA;
     if (nbatches && launch_cull(c, vt, 0, s, st) != cudaSuccess) return PC_ECUDA;
-    if (nbatches && launch_raster(c, vt, 0, s, shape, st) != cudaSuccess) return PC_ECUDA;
+    int launched = 0;
+    if (nbatches && launch_raster(c, vt, 0, s, shape, st, &launched) != cudaSuccess)
+        return PC_ECUDA;
     if (launch_resolve(c, vt, s, st) != cudaSuccess) return PC_ECUDA;
     // the device error flag and its value, for the caller to read once the
     // stream has reached this point (a copy into caller memory, no allocation)

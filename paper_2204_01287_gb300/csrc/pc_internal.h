@@ -19,12 +19,16 @@ constexpr uint32_t kMaxDim = 16384;           // width and height limit
 
 // Counter slots in Scratch::counters.
 enum : uint32_t {
-    C_ENTRIES = 0,   // draw-list entries written by the cull pass
-    C_GRAB = 1,      // entries taken by raster warps
+    C_ENTRIES = 0,   // draw-list entries written by the cull pass, from the front
+    C_GENERAL = 1,   // ... and, in one-view launches, from the back: the entries of
+                     // batches not certified for the fast path. Both counts form
+                     // one 64-bit word (one atomic reserves both).
     C_ERROR = 2,     // device error flag (nonzero = error code)
     C_ERRINFO = 3,   // first offending value
     C_GRAB_SHADE = 4,  // entries taken by high-quality shading warps
     C_GRAB_FALLBACK = 5,  // ... by the second pass of packed shading
+    C_GRAB = 6,      // entries taken by raster warps, past each warp's first
+    C_GRAB_GENERAL = 7,   // ... by the general one-view kernel
     C_COUNT = 8
 };
 
@@ -156,8 +160,9 @@ cudaError_t launch_cull(const CloudView& c, const ViewTable& vt, uint32_t view_b
                         Scratch s, cudaStream_t st);
 // LOD clouds: per node, the views whose frustum and size tests it passes.
 cudaError_t launch_lod_pass(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
+// *launched: kernels launched.
 cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, uint32_t view_base,
-                          Scratch s, RasterShape shape, cudaStream_t st);
+                          Scratch s, RasterShape shape, cudaStream_t st, int* launched);
 // High-quality shading colour pass (Sec. 3.6) over the draw list of the
 // launch, for the views with a sum buffer, and the fallback pass of packed
 // views; after launch_raster. *launched: kernels launched.

@@ -7,7 +7,7 @@
 //   k_cull      per batch and view: conservative frustum culling (Sec. 3.2) and
 //               the precision k from the projected batch extent (Sec. 3.3);
 //               surviving batches are appended, in segments, to a draw list
-//   k_raster    persistent warps take draw-list segments, load the k coordinate
+//   k_raster_*  persistent warps take draw-list segments, load the k coordinate
 //               words of 4 consecutive points with one 16-byte load per word
 //               (Sec. 3.4), decode, project (Listing 1), do the non-atomic
 //               early-depth test and atomicMin the 64-bit key; one pass serves
@@ -453,23 +453,31 @@ __global__ void __launch_bounds__(kCullThreads) k_cull(CloudView c, ViewTable vt
         const unsigned long long words = warp_sum_u64((unsigned long long)kl * (mask ? count : 0u));
         if (lane == 0 && words) atomicAdd(&sh_words, words);
     }
-    // warp-aggregated append of nseg entries
-    uint32_t incl = nseg;
+    // warp-aggregated append of nseg entries: the front list, and for one view
+    // the list from the back for batches without the fast path
+    const bool general = vt.n == 1 && !(fmask & 1u);
+    unsigned long long incl = general ? (unsigned long long)nseg << 32 : nseg;
+    const unsigned long long own = incl;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        uint32_t t = __shfl_up_sync(FULL, incl, d);
+        const unsigned long long t = __shfl_up_sync(FULL, incl, d);
         if (lane >= (uint32_t)d) incl += t;
     }
-    const uint32_t total = __shfl_sync(FULL, incl, 31);
-    uint32_t base = 0;
-    if (lane == 31 && total) base = atomicAdd(&s.counters[C_ENTRIES], total);
+    const unsigned long long total = __shfl_sync(FULL, incl, 31);
+    unsigned long long base = 0;
+    if (lane == 31 && total)
+        base = atomicAdd(reinterpret_cast<unsigned long long*>(s.counters + C_ENTRIES), total);
     base = __shfl_sync(FULL, base, 31);
-    uint64_t pos = (uint64_t)base + incl - nseg;
-    for (uint32_t g = 0; g < nseg; ++g, ++pos) {
-        if (pos >= s.capacity) {
-            raise_error(s, E_ENTRY_RANGE, (uint32_t)pos);
-            break;
-        }
+    // both lists together fit the buffer up to this warp's reservation, or none
+    // of its entries is written (later reservations do not fit then either)
+    const uint64_t end = (base >> 32) + (uint32_t)base + (total >> 32) + (uint32_t)total;
+    if (end > s.capacity) {
+        if (nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)end);
+        nseg = 0;
+    }
+    const unsigned long long at = base + incl - own;
+    uint64_t pos = general ? s.capacity - 1u - (at >> 32) : (uint32_t)at;
+    for (uint32_t g = 0; g < nseg; ++g, pos += general ? -1ll : 1ll) {
         DrawEntry e;
         e.kcodes = kcodes;
         e.view_mask = mask;
@@ -993,9 +1001,13 @@ __device__ __forceinline__ bool pixel_bracket(const FastView& fv, f2_t cxy, floa
 }
 
 // A lane's group of 4 decoded points of a certified batch in one view:
-// projection, pixel, early-depth reads and atomics.
+// projection, pixel, early-depth reads and atomics. PARTIAL: only the points in
+// the mask valid are drawn (every word of the group decodes to a point that the
+// certificate covers, so the others only cost their arithmetic).
+template <bool PARTIAL>
 __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_t (&xy)[4],
-                                                   const float (&z)[4], uint32_t g) {
+                                                   const float (&z)[4], uint32_t g,
+                                                   uint32_t valid) {
     f2_t cxy[4];
     float cw[4];
 #pragma unroll
@@ -1023,6 +1035,8 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
         pix[j] = min(by[j] * fv.width + bx[j] + fv.pixbias, fv.npix - 1u);
         w[j] = __float_as_uint(cw[j]);
         lim[j] = vis_hi[2ull * pix[j]];
+        // w is positive: a limit of 0 rejects the point
+        if (PARTIAL && !((valid >> j) & 1u)) lim[j] = 0u;
     }
     bool need = false;
 #pragma unroll
@@ -1051,27 +1065,25 @@ __device__ __forceinline__ void decode_group(const FastDec& d, const uint4& q1, 
 }
 
 // One lane's group of 4 points of a certified batch, its words given.
-template <int K>
+template <int K, bool PARTIAL>
 __device__ __forceinline__ uint32_t raster_group_fast(const FastView& fv, const FastDec& d,
                                                       const uint4& q1, const uint4& q2,
-                                                      uint32_t g) {
+                                                      uint32_t g, uint32_t valid) {
     f2_t xy[4];
     float z[4];
     decode_group<K>(d, q1, q2, xy, z);
-    return raster_decoded(fv, xy, z, g);
+    return raster_decoded<PARTIAL>(fv, xy, z, g, valid);
 }
 
-// Points [p0, p1) of a certified batch at precision K (1 or 2): whole groups
-// of 4 take the fast path, the groups of a ragged first or last step the
-// general one. A lane loads the words of its next step while it projects the
-// current one, so the load's latency hides behind that step's arithmetic. The
-// depth reads are not moved ahead: a read issued before the previous step's
-// atomics would miss their updates, and the extra atomics cost more than the
-// latency saved.
+// Points [p0, p1) of a certified batch at precision K (1 or 2). A lane loads the
+// words of its next step while it projects the current one, so the load's
+// latency hides behind that step's arithmetic. The depth reads are not moved
+// ahead: a read issued before the previous step's atomics would miss their
+// updates, and the extra atomics cost more than the latency saved.
 template <int K, bool STREAM>
-__device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const ViewConst& vc,
-                                                 const FastView& fv, const pc_batch& bt,
-                                                 uint32_t p0, uint32_t p1, uint32_t lane) {
+__device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const FastView& fv,
+                                                 const pc_batch& bt, uint32_t p0, uint32_t p1,
+                                                 uint32_t lane) {
     uint32_t n_atom = 0;
     uint32_t base = p0 & ~3u;
     if (lane == 0 && p1 > base) {
@@ -1079,21 +1091,25 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const ViewC
         prefetch_l2(c.w1 + base, bytes);
         if (K >= 2) prefetch_l2(c.w2 + base, bytes);
     }
-    if (base != p0 && base < p1) {
-        const uint32_t g = base + 4u * lane;
-        if (g < p1) {
-            uint32_t valid = 0;
+    const FastDec d = make_fast_dec<K>(bt);
+    // the ragged first and last steps
+    auto partial = [&](uint32_t g) {
+        if (g >= p1) return;
+        uint32_t valid = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) valid |= (uint32_t)(g + j >= p0 && g + j < p1) << j;
-            n_atom += raster_group<K, STREAM, true>(c, vc, make_dec_const(bt, K), g, valid);
-        }
+        for (int j = 0; j < 4; ++j) valid |= (uint32_t)(g + j >= p0 && g + j < p1) << j;
+        const uint4 q1 = ld_words<STREAM>(c.w1 + g);
+        const uint4 q2 = K >= 2 ? ld_words<STREAM>(c.w2 + g) : make_uint4(0, 0, 0, 0);
+        n_atom += raster_group_fast<K, true>(fv, d, q1, q2, g, valid);
+    };
+    if (base != p0 && base < p1) {
+        partial(base + 4u * lane);
         base += 128u;
     }
     if (base + 128u <= p1) {
         // whole steps: the next step's words are loaded while the current one
         // is projected; the last step is peeled so that the loop carries no
         // bounds test, and two steps are unrolled
-        const FastDec d = make_fast_dec<K>(bt);
         const uint32_t nsteps = (p1 - base) >> 7;
         uint32_t g = base + 4u * lane;
         const uint32_t* a1 = c.w1 + g;
@@ -1110,21 +1126,13 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const ViewC
                 a2 += 128;
                 n2 = ld_words<STREAM>(a2);
             }
-            n_atom += raster_group_fast<K>(fv, d, q1, q2, g);
+            n_atom += raster_group_fast<K, false>(fv, d, q1, q2, g, 0xFu);
             g += 128u;
         }
-        n_atom += raster_group_fast<K>(fv, d, n1, n2, g);
+        n_atom += raster_group_fast<K, false>(fv, d, n1, n2, g, 0xFu);
         base += nsteps << 7;
     }
-    if (base < p1) {
-        const uint32_t g = base + 4u * lane;
-        if (g < p1) {
-            uint32_t valid = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) valid |= (uint32_t)(g + j < p1) << j;
-            n_atom += raster_group<K, STREAM, true>(c, vc, make_dec_const(bt, K), g, valid);
-        }
-    }
+    if (base < p1) partial(base + 4u * lane);
     return n_atom;
 }
 
@@ -1180,7 +1188,7 @@ __device__ __forceinline__ void segment_fast_views(const CloudView& c, const Vie
             decode_group<K>(d, q1, q2, xy, z);
             for (uint32_t mm = vmask; mm; mm &= mm - 1) {
                 const uint32_t v = __ffs(mm) - 1;
-                const uint32_t n = raster_decoded(make_fast_view(vt.v[v]), xy, z, g);
+                const uint32_t n = raster_decoded<false>(make_fast_view(vt.v[v]), xy, z, g, 0xFu);
                 if (n) atomicAdd(&sh_atom[v], n);
             }
         }
@@ -1244,8 +1252,8 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
             f2_t xy[4];
             float z[4];
             decode_group<K>(d, q1, q2, xy, z);
-            if (vmask & 1u) na0 += raster_decoded(make_fast_view(vt.v[0]), xy, z, g);
-            if (vmask & 2u) na1 += raster_decoded(make_fast_view(vt.v[1]), xy, z, g);
+            if (vmask & 1u) na0 += raster_decoded<false>(make_fast_view(vt.v[0]), xy, z, g, 0xFu);
+            if (vmask & 2u) na1 += raster_decoded<false>(make_fast_view(vt.v[1]), xy, z, g, 0xFu);
         };
         for (uint32_t st = 1; st < nsteps; ++st) {
             const uint4 q1 = n1, q2 = n2;
@@ -1274,25 +1282,35 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
 
 constexpr int kRasterThreads = 256;
 
-__device__ __forceinline__ bool next_entry(const Scratch& s, uint32_t n_entries, uint32_t lane,
-                                           DrawEntry& e) {
-    uint32_t e_idx = 0;
-    if (lane == 0) e_idx = atomicAdd(&s.counters[C_GRAB], 1u);
-    e_idx = __shfl_sync(FULL, e_idx, 0);
-    if (e_idx >= n_entries || e_idx >= s.capacity) return false;
-    e = s.entries[e_idx];
-    return true;
+// How the persistent warps share a list of n entries: a warp's first entry is
+// its own index in the grid, and only the entries past the grid's warps are
+// taken from a counter. A list that the grid covers in one round takes no
+// atomic; with one atomic per entry and one more per warp to see the end,
+// thousands of returning atomics on one address were the bound of small frames
+// (raster pass of an LOD frame of 1.3M points 26 us, 17 us this way).
+__device__ __forceinline__ uint32_t grid_warps() { return gridDim.x * (blockDim.x >> 5); }
+__device__ __forceinline__ uint32_t first_entry() {
+    return __shfl_sync(FULL, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), 0);
+}
+__device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counter, uint32_t n,
+                                               uint32_t lane) {
+    uint32_t i = n;
+    if (lane == 0 && n > grid_warps()) i = grid_warps() + atomicAdd(&s.counters[counter], 1u);
+    return __shfl_sync(FULL, i, 0);
 }
 
-// One segment for one view at its precision k; certified batches (fast) at
-// k <= 2 take the fast path.
+// Lengths of the draw list's two parts; none when they overflowed the buffer.
+__device__ __forceinline__ void entry_counts(const Scratch& s, uint32_t& front, uint32_t& back) {
+    front = s.counters[C_ENTRIES];
+    back = s.counters[C_GENERAL];
+    if ((uint64_t)front + back > s.capacity) front = back = 0;
+}
+
+// One segment for one view at its precision k on the general path.
 template <bool STREAM>
 __device__ __forceinline__ uint32_t segment_k(const CloudView& c, const ViewConst& vc,
-                                              const FastView& fv, const pc_batch& bt, int k,
-                                              bool fast, uint32_t p0, uint32_t p1,
-                                              uint32_t lane) {
-    if (fast && k == 1) return segment_fast<1, STREAM>(c, vc, fv, bt, p0, p1, lane);
-    if (fast && k == 2) return segment_fast<2, STREAM>(c, vc, fv, bt, p0, p1, lane);
+                                              const pc_batch& bt, int k, uint32_t p0,
+                                              uint32_t p1, uint32_t lane) {
     const DecConst d = make_dec_const(bt, k);
     if (k == 1) return segment<1, STREAM>(c, vc, d, p0, p1, lane);
     if (k == 2) return segment<2, STREAM>(c, vc, d, p0, p1, lane);
@@ -1306,26 +1324,59 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
         atomicAdd(&s.stats[(uint64_t)view * S_COUNT + S_ATOMICS], (unsigned long long)t);
 }
 
-// One view per launch: persistent warps take draw-list segments. Five blocks
-// of 256 threads per SM (48 registers): the depth reads' latency is hidden by
-// other warps, and more warps hide more of it.
-__global__ void __launch_bounds__(kRasterThreads, 5) k_raster1(CloudView c, ViewTable vt,
-                                                           uint32_t view_base, Scratch s) {
+// One view per launch: two kernels, so that neither path's registers burden the
+// other. The certified entries (the draw list's front) go to k_raster_fast, the
+// others (its back) to k_raster_general, launched just before it. The fast
+// kernel starts as soon as the general one's blocks have started
+// (programmatic launch): both only read what the cull pass wrote and update the
+// view by atomics, so they may run side by side. In one kernel at 48 registers
+// the general path spilled (a 100M-point fly-through frame's raster pass took
+// 99 us, 74 us with two kernels); at 64 registers both paths fit, but the fast
+// path wants the fifth block (2B points: 3.43 ms against 3.30 ms).
+
+// Five blocks of 256 threads per SM (48 registers): the depth reads' latency is
+// hidden by other warps, and more warps hide more of it.
+__global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c, ViewTable vt,
+                                                               uint32_t view_base, Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_entries = s.counters[C_ENTRIES];
-    const ViewConst vc = make_view_const(vt.v[0]);
+    uint32_t n_entries, n_back;
+    entry_counts(s, n_entries, n_back);
     const FastView fv = make_fast_view(vt.v[0]);
     uint32_t n_atom = 0;
-    DrawEntry e;
-    while (next_entry(s, n_entries, lane, e)) {
+    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+        const DrawEntry e = s.entries[i];
+        if (e.batch >= c.n_batches) {
+            if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
+            continue;
+        }
+        const pc_batch bt = c.batches[e.batch];
+        const uint32_t p0 = bt.first + e.seg_first, p1 = p0 + e.seg_count;
+        n_atom += (e.kcodes & 3u) == 1u ? segment_fast<1, true>(c, fv, bt, p0, p1, lane)
+                                        : segment_fast<2, true>(c, fv, bt, p0, p1, lane);
+    }
+    flush_atomics(s, view_base, n_atom, lane);
+    // what follows in the stream waits for this kernel: it ends after the other
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView c, ViewTable vt,
+                                                                  uint32_t view_base, Scratch s) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const uint32_t lane = threadIdx.x & 31;
+    uint32_t n_front, n_entries;
+    entry_counts(s, n_front, n_entries);
+    const ViewConst vc = make_view_const(vt.v[0]);
+    uint32_t n_atom = 0;
+    for (uint32_t i = first_entry(); i < n_entries;
+         i = next_entry(s, C_GRAB_GENERAL, n_entries, lane)) {
+        const DrawEntry e = s.entries[s.capacity - 1u - i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
         }
         const pc_batch bt = c.batches[e.batch];
         const uint32_t p0 = bt.first + e.seg_first;
-        n_atom += segment_k<true>(c, vc, fv, bt, (int)(e.kcodes & 3u), e.fast_mask & 1u, p0,
-                                  p0 + e.seg_count, lane);
+        n_atom += segment_k<true>(c, vc, bt, (int)(e.kcodes & 3u), p0, p0 + e.seg_count, lane);
     }
     flush_atomics(s, view_base, n_atom, lane);
 }
@@ -1336,10 +1387,11 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster1(CloudView c, View
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, ViewTable vt,
                                                            uint32_t view_base, Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_entries = s.counters[C_ENTRIES];
+    uint32_t n_entries, n_back;
+    entry_counts(s, n_entries, n_back);
     uint32_t na0 = 0, na1 = 0;
-    DrawEntry e;
-    while (next_entry(s, n_entries, lane, e)) {
+    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+        const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
@@ -1359,11 +1411,11 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, View
         if (fast2) segment_fast_pair<2>(c, vt, fast2, bt, p0, p1, lane, na0, na1);
         const uint32_t rest = e.view_mask & ~(fast1 | fast2);
         if (rest & 1u)
-            na0 += segment_k<false>(c, make_view_const(vt.v[0]), make_fast_view(vt.v[0]), bt,
-                                    (int)(e.kcodes & 3u), false, p0, p1, lane);
+            na0 += segment_k<false>(c, make_view_const(vt.v[0]), bt, (int)(e.kcodes & 3u), p0, p1,
+                                    lane);
         if (rest & 2u)
-            na1 += segment_k<false>(c, make_view_const(vt.v[1]), make_fast_view(vt.v[1]), bt,
-                                    (int)((e.kcodes >> 2) & 3u), false, p0, p1, lane);
+            na1 += segment_k<false>(c, make_view_const(vt.v[1]), bt, (int)((e.kcodes >> 2) & 3u),
+                                    p0, p1, lane);
     }
     flush_atomics(s, view_base, na0, lane);
     flush_atomics(s, view_base + 1, na1, lane);
@@ -1380,9 +1432,10 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, View
     for (uint32_t i = threadIdx.x; i < kMaxViewsPerLaunch; i += blockDim.x) sh_atom[i] = 0;
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_entries = s.counters[C_ENTRIES];
-    DrawEntry e;
-    while (next_entry(s, n_entries, lane, e)) {
+    uint32_t n_entries, n_back;
+    entry_counts(s, n_entries, n_back);
+    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+        const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
@@ -1402,9 +1455,8 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, View
         for (uint32_t mm = e.view_mask & ~(fast1 | fast2); mm; mm &= mm - 1) {
             const uint32_t v = __ffs(mm) - 1;
             const ViewConst vc = make_view_const(vt.v[v]);
-            const FastView fv = make_fast_view(vt.v[v]);
-            const uint32_t n = segment_k<false>(c, vc, fv, bt, (int)((e.kcodes >> (2 * v)) & 3u),
-                                                false, p0, p0 + e.seg_count, lane);
+            const uint32_t n = segment_k<false>(c, vc, bt, (int)((e.kcodes >> (2 * v)) & 3u), p0,
+                                                p0 + e.seg_count, lane);
             const uint32_t t = __reduce_add_sync(FULL, n);
             if (lane == 0 && t) atomicAdd(&sh_atom[v], t);
         }
@@ -1782,14 +1834,12 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, uin
     for (uint32_t i = threadIdx.x; i < kMaxViewsPerLaunch; i += blockDim.x) sh_blend[i] = 0;
     __syncthreads();
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t n_entries = s.counters[C_ENTRIES];
-    unsigned int* grab = &s.counters[FALLBACK ? C_GRAB_FALLBACK : C_GRAB_SHADE];
-    for (;;) {
-        uint32_t e_idx = 0;
-        if (lane == 0) e_idx = atomicAdd(grab, 1u);
-        e_idx = __shfl_sync(FULL, e_idx, 0);
-        if (e_idx >= n_entries || e_idx >= s.capacity) break;
-        const DrawEntry e = s.entries[e_idx];
+    uint32_t n_front, n_entries;
+    entry_counts(s, n_front, n_entries);
+    n_entries += n_front;
+    for (uint32_t i = first_entry(); i < n_entries;
+         i = next_entry(s, FALLBACK ? C_GRAB_FALLBACK : C_GRAB_SHADE, n_entries, lane)) {
+        const DrawEntry e = s.entries[i < n_front ? i : s.capacity - 1u - (i - n_front)];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
@@ -1996,20 +2046,33 @@ int raster_occupancy(int threads_per_block, uint32_t nviews) {
     cudaError_t e =
         nviews > 2    ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_rasterN, threads_per_block, 0)
         : nviews == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_raster2, threads_per_block, 0)
-                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_raster1, threads_per_block, 0);
+                      : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_raster_fast, threads_per_block, 0);
     if (e != cudaSuccess) return 1;
     return nb > 0 ? nb : 1;
 }
 
 cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
-                          RasterShape shape, cudaStream_t st) {
+                          RasterShape shape, cudaStream_t st, int* launched) {
     int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
     threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
-    int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
+    const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
+    *launched = vt.n == 1 ? 2 : 1;
     if (vt.n > 2) k_rasterN<<<blocks, threads, 0, st>>>(c, vt, view_base, s);
     else if (vt.n == 2) k_raster2<<<blocks, threads, 0, st>>>(c, vt, view_base, s);
-    else k_raster1<<<blocks, threads, 0, st>>>(c, vt, view_base, s);
-    return cudaGetLastError();
+    if (vt.n != 1) return cudaGetLastError();
+    k_raster_general<<<num_sms() * 4, kRasterThreads, 0, st>>>(c, vt, view_base, s);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cfg.attrs = &early;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, vt, view_base, s);
 }
 
 template <int LAYOUTS>
