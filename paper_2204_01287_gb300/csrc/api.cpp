@@ -70,7 +70,6 @@ Slot::~Slot() {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
     cudaFree(scratch.entries);
     cudaFree(scratch.counters);
-    cudaFree(scratch.stats);
     cudaFree(scratch.lod_sel);
     cudaFree(hqs_accum);
     cudaFree(host_vis);
@@ -78,23 +77,30 @@ Slot::~Slot() {
 }
 
 pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
-    // each buffer on its own, so a failed allocation is retried by the next call
+    // counters, sums and statistics are one allocation, the others each on its
+    // own, so a failed allocation is retried by the next call
     if (!s.scratch.counters) {
-        cudaError_t e = cudaMalloc(&s.scratch.counters, sizeof(uint32_t) * C_COUNT);
-        if (e != cudaSuccess) {
-            s.scratch.counters = nullptr;
-            return cuda_fail(e, "scratch counters");
-        }
-        cudaMemsetAsync(s.scratch.counters, 0, sizeof(uint32_t) * C_COUNT, s.stream);
+        const size_t words = C_COUNT / 2 + (kMaxViewsPerLaunch + kMaxViewsPerRender) * S_COUNT;
+        unsigned long long* p = nullptr;
+        cudaError_t e = cudaMalloc(&p, words * sizeof(unsigned long long));
+        if (e != cudaSuccess) return cuda_fail(e, "scratch counters");
+        s.scratch.counters = reinterpret_cast<uint32_t*>(p);
+        s.scratch.acc = p + C_COUNT / 2;
+        s.scratch.stats = s.scratch.acc + kMaxViewsPerLaunch * S_COUNT;
+        cudaMemsetAsync(p, 0, words * sizeof(unsigned long long), s.stream);
     }
-    if (!s.scratch.stats) {
-        const size_t bytes = sizeof(unsigned long long) * kMaxViewsPerRender * S_COUNT;
-        cudaError_t e = cudaMalloc(&s.scratch.stats, bytes);
-        if (e != cudaSuccess) {
-            s.scratch.stats = nullptr;
-            return cuda_fail(e, "scratch stats");
-        }
-        cudaMemsetAsync(s.scratch.stats, 0, bytes, s.stream);
+    if (s.unclean) {
+        // a frame whose launches failed part-way: its last pass did not leave
+        // the counters (the error words apart) and sums at zero
+        cudaError_t e = cudaMemsetAsync(s.scratch.acc, 0,
+                                        sizeof(unsigned long long) * kMaxViewsPerLaunch * S_COUNT, s.stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(s.scratch.counters, 0, sizeof(uint32_t) * C_ERROR, s.stream);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(s.scratch.counters + C_ERRINFO + 1, 0,
+                                sizeof(uint32_t) * (C_COUNT - C_ERRINFO - 1), s.stream);
+        if (e != cudaSuccess) return cuda_fail(e, "scratch reset");
+        s.unclean = false;
     }
     if (entries > s.scratch.capacity) {
         cudaStreamSynchronize(s.stream);
@@ -110,7 +116,7 @@ pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
         cudaFree(s.scratch.lod_sel);
         s.scratch.lod_sel = nullptr;
         s.lod_capacity = 0;
-        cudaError_t e = cudaMalloc(&s.scratch.lod_sel, nodes * sizeof(uint32_t));
+        cudaError_t e = cudaMalloc(&s.scratch.lod_sel, nodes * sizeof(LodSel));
         if (e != cudaSuccess) return cuda_fail(e, "lod selection");
         s.lod_capacity = nodes;
     }
@@ -257,38 +263,36 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         cudaError_t e = cudaSuccess;
         if (fo.resolve_only) {
             if (fe) for (int i = 1; i < 5; ++i) cudaEventRecord(fe->ev[i], st);
-            e = launch_resolve(cv, vt, slot->scratch, st);
+            e = launch_resolve(cv, vt, base, slot->scratch, false, st);
             if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
             if (fe) cudaEventRecord(fe->ev[5], st);
             launches += 1;
             continue;
         }
-        e = launch_clear(vt, base, slot->scratch, st);
-        if (e != cudaSuccess) return cuda_fail(e, "clear launch");
-        if (fe) cudaEventRecord(fe->ev[1], st);
+        if (fe) cudaEventRecord(fe->ev[1], st);   // the clear runs beside the culling
+        e = launch_begin(cv, vt, slot->scratch, st);
+        if (e != cudaSuccess) return cuda_fail(e, "cull launch");
         if (cl.is_lod) {
-            e = launch_lod_pass(cv, vt, slot->scratch, st);
+            e = launch_lod_append(cv, vt, slot->scratch, st);
             if (e != cudaSuccess) return cuda_fail(e, "LOD selection launch");
             launches += 1;
         }
-        e = launch_cull(cv, vt, base, slot->scratch, st);
-        if (e != cudaSuccess) return cuda_fail(e, "cull launch");
         if (fe) cudaEventRecord(fe->ev[2], st);
         int raster_kernels = 0;
-        e = launch_raster(cv, vt, base, slot->scratch, shape, st, &raster_kernels);
+        e = launch_raster(cv, vt, slot->scratch, shape, st, &raster_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "raster launch");
         if (fe) cudaEventRecord(fe->ev[3], st);
         if (shade) {
             int nk = 0;
-            e = launch_shade(cv, vt, base, slot->scratch, shape, st, &nk);
+            e = launch_shade(cv, vt, slot->scratch, shape, st, &nk);
             if (e != cudaSuccess) return cuda_fail(e, "shading launch");
             launches += nk;
         }
         if (fe) cudaEventRecord(fe->ev[4], st);
-        e = launch_resolve(cv, vt, slot->scratch, st);
+        e = launch_resolve(cv, vt, base, slot->scratch, true, st);
         if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
         if (fe) cudaEventRecord(fe->ev[5], st);
-        launches += 3 + raster_kernels;
+        launches += 2 + raster_kernels;
         raster_launches += 1;
     }
     return PC_OK;
@@ -363,6 +367,7 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
     rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, fo);
+    if (rc != PC_OK) slot->unclean = true;
     if (graph) {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(st, &g);

@@ -24,13 +24,14 @@ constexpr uint32_t kNoAllocMaxSegment = 1u << 20;
 struct NoAllocLayout {
     DrawEntry entries[kNoAllocEntries];
     uint32_t counters[C_COUNT];
+    unsigned long long acc[S_COUNT];
     unsigned long long stats[S_COUNT];
 };
-// counters and stats are cleared by one memset, so stats must follow counters
+// counters and sums are cleared by one memset, so acc must follow counters
 // with no gap
-static_assert(offsetof(NoAllocLayout, stats) ==
+static_assert(offsetof(NoAllocLayout, acc) ==
                   offsetof(NoAllocLayout, counters) + sizeof(uint32_t) * C_COUNT,
-              "stats directly follows counters");
+              "acc directly follows counters");
 
 // About 4 MB per device, held by every GPU that loads the library until exit.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(NoAllocLayout)];
@@ -99,11 +100,12 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     s.entries = L->entries;
     s.capacity = kNoAllocEntries;
     s.counters = L->counters;
+    s.acc = L->acc;
     s.stats = L->stats;
     s.lod_sel = nullptr;
-    // the array keeps the previous call's contents: counters and statistics
+    // the array keeps the previous call's contents: counters and sums
     // (including the error flag) start from zero every call
-    if (cudaMemsetAsync(L->counters, 0, sizeof L->counters + sizeof L->stats, st) != cudaSuccess)
+    if (cudaMemsetAsync(L->counters, 0, sizeof L->counters + sizeof L->acc, st) != cudaSuccess)
         return PC_ECUDA;
 
     CloudView c;
@@ -133,12 +135,11 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     RasterShape shape;
     shape.threads_per_block = 256;
     shape.blocks = 0;   // one resident wave
-    if (launch_clear(vt, 0, s, st) != cudaSuccess) return PC_ECUDA;
-    if (nbatches && launch_cull(c, vt, 0, s, st) != cudaSuccess) return PC_ECUDA;
+    if (launch_begin(c, vt, s, st) != cudaSuccess) return PC_ECUDA;
     int launched = 0;
-    if (nbatches && launch_raster(c, vt, 0, s, shape, st, &launched) != cudaSuccess)
+    if (nbatches && launch_raster(c, vt, s, shape, st, &launched) != cudaSuccess)
         return PC_ECUDA;
-    if (launch_resolve(c, vt, s, st) != cudaSuccess) return PC_ECUDA;
+    if (launch_resolve(c, vt, 0, s, true, st) != cudaSuccess) return PC_ECUDA;
     // the device error flag and its value, for the caller to read once the
     // stream has reached this point (a copy into caller memory, no allocation)
     if (device_error && cudaMemcpyAsync(device_error, L->counters + C_ERROR, 2 * sizeof(uint32_t),

@@ -61,6 +61,7 @@ struct Slot {
     uint64_t* host_vis = nullptr;     // pc_render_host framebuffers
     uint32_t* host_rgba = nullptr;
     uint64_t host_pixels = 0;
+    bool unclean = false;           // a frame's launches failed part-way (see ensure_capacity)
     uint32_t last_nviews = 0;
     uint64_t last_total_batches = 0;
     std::map<uint64_t, cudaGraphExec_t> graphs;   // replayable frames by launch layout

@@ -29,7 +29,7 @@ enum : uint32_t {
     C_GRAB_FALLBACK = 5,  // ... by the second pass of packed shading
     C_GRAB = 6,      // entries taken by raster warps, past each warp's first
     C_GRAB_GENERAL = 7,   // ... by the general one-view kernel
-    C_COUNT = 8
+    C_COUNT = 8       // even: the scratch sums follow the counters
 };
 
 // Per-view statistics slots in Scratch::stats (uint64 each).
@@ -137,13 +137,23 @@ struct DrawEntry {
 };
 static_assert(sizeof(DrawEntry) == 32, "draw-list entries are 32 bytes");
 
+// What the views of a launch make of a batch: bit v of mask: view v draws it (for
+// an LOD node: it passes view v); its precisions and certificates as in DrawEntry.
+struct LodSel {
+    unsigned long long kcodes;
+    uint32_t mask, fast;
+};
+
 // Per-stream scratch memory (device).
 struct Scratch {
     DrawEntry* entries;
     uint64_t capacity;    // entries
     uint32_t* counters;   // C_COUNT
-    unsigned long long* stats;  // kMaxViewsPerRender * S_COUNT
-    uint32_t* lod_sel;    // LOD: per node, bit v = node passes view v of the launch
+    unsigned long long* stats;  // kMaxViewsPerRender * S_COUNT: the last frame's
+    unsigned long long* acc;    // kMaxViewsPerLaunch * S_COUNT: sums of the launch in
+                                // progress. acc and counters (the error words apart)
+                                // are zero between launches; k_resolve leaves them so
+    LodSel* lod_sel;      // LOD: per node
 };
 
 // Launch-shape knobs for the raster kernel.
@@ -154,22 +164,21 @@ struct RasterShape {
 
 // ---- kernel launchers (raster.cu) ----------------------------------------
 
-cudaError_t launch_clear(const ViewTable& vt, uint32_t view_base, Scratch s,
-                         cudaStream_t st);
-cudaError_t launch_cull(const CloudView& c, const ViewTable& vt, uint32_t view_base,
-                        Scratch s, cudaStream_t st);
-// LOD clouds: per node, the views whose frustum and size tests it passes.
-cudaError_t launch_lod_pass(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
+// Clears the views' buffers, tests every batch against every view and, for a plain
+// cloud, writes the draw list; for an LOD cloud launch_lod_append writes it.
+cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
+cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
 // *launched: kernels launched.
-cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, uint32_t view_base,
-                          Scratch s, RasterShape shape, cudaStream_t st, int* launched);
+cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s, RasterShape shape, cudaStream_t st, int* launched);
 // High-quality shading colour pass (Sec. 3.6) over the draw list of the
 // launch, for the views with a sum buffer, and the fallback pass of packed
 // views; after launch_raster. *launched: kernels launched.
-cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
+cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, Scratch s,
                          RasterShape shape, cudaStream_t st, int* launched);
-cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, Scratch s,
-                           cudaStream_t st);
+// publish: the launch's statistics become stats[view_base ..] and the scratch
+// counters return to zero (every launch but a resolve alone).
+cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
+                           bool publish, cudaStream_t st);
 // dst[i] = min(dst[i], src[i]) over n keys (both 16-byte aligned).
 cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cudaStream_t st);
 

@@ -1,12 +1,11 @@
 // raster.cu — sm_103a kernels of the point rasterizer.
 //
-//   k_clear     visibility buffers <- all ones (and shading sums <- 0); scratch
-//               counters <- 0
-//   k_lod_pass  LOD clouds: per node and view, frustum, projected extent and
-//               (foveated) threshold (Sec. 3.5, 3.7)
-//   k_cull      per batch and view: conservative frustum culling (Sec. 3.2) and
-//               the precision k from the projected batch extent (Sec. 3.3);
-//               surviving batches are appended, in segments, to a draw list
+//   k_begin     visibility buffers <- empty (and shading sums <- 0), and per batch
+//               and view: conservative frustum culling (Sec. 3.2) and the precision
+//               k from the projected batch extent (Sec. 3.3); surviving batches are
+//               appended, in segments, to a draw list. LOD clouds: frustum, projected
+//               extent and (foveated) threshold of every node (Sec. 3.5, 3.7)
+//   k_lod_append  LOD clouds: the nodes whose ancestors pass too, to the draw list
 //   k_raster_*  persistent warps take draw-list segments, load the k coordinate
 //               words of 4 consecutive points with one 16-byte load per word
 //               (Sec. 3.4), decode, project (Listing 1), do the non-atomic
@@ -38,37 +37,24 @@ __device__ __forceinline__ void raise_error(Scratch s, uint32_t code, uint32_t i
     if (atomicCAS(&s.counters[C_ERROR], 0u, code) == 0u) s.counters[C_ERRINFO] = info;
 }
 
-// ---- k_clear -----------------------------------------------------------------
+// ---- clear --------------------------------------------------------------------
 
-__global__ void k_clear(ViewTable vt, uint32_t view_base, Scratch s) {
-    const uint32_t v = blockIdx.y;
-    if (blockIdx.x == 0 && v == 0) {
-        if (threadIdx.x < C_COUNT && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
-            s.counters[threadIdx.x] = 0u;
-        for (uint32_t i = threadIdx.x; i < vt.n * S_COUNT; i += blockDim.x)
-            s.stats[(uint64_t)view_base * S_COUNT + i] = 0ull;
-    }
-    if (v >= vt.n) return;
-    const ViewParams& vp = vt.v[v];
+// Part `part` of `parts` of view v's buffers: visibility keys <- empty, shading
+// sums <- 0. 16-byte stores (vis is 16-byte aligned, checked on the host).
+__device__ __forceinline__ void clear_view(const ViewParams& vp, uint32_t part, uint32_t parts) {
     const uint64_t npix = (uint64_t)vp.width * vp.height;
-    // 16-byte stores; vis is 16-byte aligned (checked on the host)
+    const uint64_t t0 = (uint64_t)part * blockDim.x + threadIdx.x, step = (uint64_t)parts * blockDim.x;
     ulonglong2* p2 = reinterpret_cast<ulonglong2*>(vp.vis);
-    const uint64_t n2 = npix / 2;
     const unsigned long long empty = empty_key(vp.flags);
     const ulonglong2 ones = make_ulonglong2(empty, empty);
-    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        p2[i] = ones;
-    if ((npix & 1) && blockIdx.x == 0 && threadIdx.x == 0) vp.vis[npix - 1] = empty;
+    for (uint64_t i = t0; i < npix / 2; i += step) p2[i] = ones;
+    if ((npix & 1) && t0 == 0) vp.vis[npix - 1] = empty;
     if (vp.accum) {
-        // high-quality shading sums <- 0; each view's region is a whole number
-        // of 16-byte words
+        // each view's region is a whole number of 16-byte words
         ulonglong2* a2 = reinterpret_cast<ulonglong2*>(vp.accum);
         const uint64_t na = (hqs_clear_words(vp.flags, npix) + 1) / 2;
         const ulonglong2 zero = make_ulonglong2(0ull, 0ull);
-        for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < na;
-             i += (uint64_t)gridDim.x * blockDim.x)
-            a2[i] = zero;
+        for (uint64_t i = t0; i < na; i += step) a2[i] = zero;
     }
 }
 
@@ -86,39 +72,6 @@ __device__ __forceinline__ float to_pixel(float c, float w, float W) {
     return __fmul_rn(__fadd_rn(__fmul_rn(__fdiv_rn(c, w), 0.5f), 0.5f), W);
 }
 
-// Spread of the 8 projected box corners' unfloored pixel coordinates, with
-// the same binary32 operations as a point; false when a corner has w <= 0.
-__device__ bool corner_box(const pc_batch& b, const ViewParams& v, float& fmin0, float& fmax0,
-                           float& fmin1, float& fmax1) {
-    float hi[3];
-    for (int a = 0; a < 3; ++a) hi[a] = __fadd_rn(b.min[a], b.size[a]);
-    fmin0 = fmax0 = fmin1 = fmax1 = 0.f;
-    const float W = (float)v.width, H = (float)v.height;
-#pragma unroll 1
-    for (int c = 0; c < 8; ++c) {
-        float x = (c & 1) ? hi[0] : b.min[0];
-        float y = (c & 2) ? hi[1] : b.min[1];
-        float z = (c & 4) ? hi[2] : b.min[2];
-        float cw = clip_row(v.m, 3, x, y, z);
-        if (!(cw > 0.0f)) return false;
-        float f0 = to_pixel(clip_row(v.m, 0, x, y, z), cw, W);
-        float f1 = to_pixel(clip_row(v.m, 1, x, y, z), cw, H);
-        if (c == 0 || f0 < fmin0) fmin0 = f0;
-        if (c == 0 || f0 > fmax0) fmax0 = f0;
-        if (c == 0 || f1 < fmin1) fmin1 = f1;
-        if (c == 0 || f1 > fmax1) fmax1 = f1;
-    }
-    return true;
-}
-
-__device__ bool corner_extent(const pc_batch& b, const ViewParams& v, float& ex, float& ey) {
-    float fmin0, fmax0, fmin1, fmax1;
-    if (!corner_box(b, v, fmin0, fmax0, fmin1, fmax1)) return false;
-    ex = __fsub_rn(fmax0, fmin0);
-    ey = __fsub_rn(fmax1, fmin1);
-    return true;
-}
-
 // Sec. 3.7 rings of a screen position: 0 within a third of the half-diagonal
 // from the view centre, 1 within two thirds, else 2 (binary32, fixed order).
 __device__ __forceinline__ int ring_of(float x, float y, uint32_t width, uint32_t height) {
@@ -130,19 +83,6 @@ __device__ __forceinline__ int ring_of(float x, float y, uint32_t width, uint32_
     if (d9 < r2) return 0;
     if (d9 < __fmul_rn(4.0f, r2)) return 1;
     return 2;
-}
-
-// Sec. 3.3: smallest k whose cells are below the threshold, from the extent
-// of the 8 projected box corners; 3 when a corner is not in front of the eye.
-__device__ int select_k(const pc_batch& b, const ViewParams& v, float T) {
-    const uint32_t fk = (v.flags & PC_VIEW_K_MASK) >> 4;
-    if (fk >= 1) return (int)fk;
-    float ex, ey;
-    if (!corner_extent(b, v, ex, ey)) return 3;
-    if (ex < T && ey < T) return 1;
-    const float T2 = __fmul_rn(T, 1024.0f);
-    if (ex < T2 && ey < T2) return 2;
-    return 3;
 }
 
 // Conservative culling: the batch is dropped only if, for one clip plane, a
@@ -206,13 +146,7 @@ __device__ bool cull_batch_exact(const pc_batch& b, const ViewParams& v) {
     return false;
 }
 
-// The same five tests in binary32 first. Each test value t approximates the
-// exact value R of its expression within about 10 * 2^-24 of the magnitude M
-// of its terms, and the binary64 value within about 10 * 2^-53 M, so when
-// |t| > 2^-16 M both have the sign of R and the decision equals the binary64
-// one. Inside that band, or when a magnitude is not finite or below 2^-90
-// (where products could lose bits to underflow), the binary64 code decides.
-// Returns 1 culled, 0 not culled, -1 undecided.
+// The rows of the tests in binary32.
 __device__ __forceinline__ float row_max32(const float r[4], const float lo[3], const float hi[3]) {
     float s = r[3];
 #pragma unroll
@@ -233,267 +167,367 @@ __device__ __forceinline__ float row_mag32(const float r[4], const float lo[3], 
     return s;
 }
 
-__device__ __forceinline__ int cull_batch_fast(const pc_batch& b, const ViewParams& v) {
-    const float g = 6.0f * 0x1.0p-24f;
-    const float e1 = 1.0f + 0x1.0p-10f;
-    const float band = 0x1.0p-16f;
-    float lo[3], hi[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        lo[a] = b.min[a];
-        hi[a] = __fadd_rn(b.min[a], b.size[a]);
-    }
-    const float* m = v.m;
-    const float X[4] = {m[0], m[4], m[8], m[12]};
-    const float Y[4] = {m[1], m[5], m[9], m[13]};
-    const float Wr[4] = {m[3], m[7], m[11], m[15]};
-    const float bx = row_mag32(X, lo, hi), by = row_mag32(Y, lo, hi), bw = row_mag32(Wr, lo, hi);
-    const float mag_x = __fadd_rn(bx, __fmul_rn(e1, bw)), mag_y = __fadd_rn(by, __fmul_rn(e1, bw));
-    if (!(bw <= 0x1.0p100f) || !(mag_x <= 0x1.0p100f) || !(mag_y <= 0x1.0p100f)) return -1;
-    if (!(bw >= 0x1.0p-90f) || !(mag_x >= 0x1.0p-90f) || !(mag_y >= 0x1.0p-90f)) return -1;
-    // each test: culled when t < 0 (t <= 0 for the w plane), decided when |t| > band M
-    bool undecided = false, culled = false;
-    auto test = [&](float t, float mag) {
-        const float lim = __fmul_rn(band, mag);
-        if (t < -lim) culled = true;
-        else if (!(t > lim)) undecided = true;
-    };
-    test(__fadd_rn(row_max32(Wr, lo, hi), __fmul_rn(g, bw)), bw);
-    float sp[4], sm[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        sp[a] = __fadd_rn(X[a], __fmul_rn(e1, Wr[a]));
-        sm[a] = __fsub_rn(X[a], __fmul_rn(e1, Wr[a]));
-    }
-    const float mx = __fmul_rn(g, mag_x);
-    test(__fadd_rn(row_max32(sp, lo, hi), mx), mag_x);
-    test(-__fsub_rn(row_min32(sm, lo, hi), mx), mag_x);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-        sp[a] = __fadd_rn(Y[a], __fmul_rn(e1, Wr[a]));
-        sm[a] = __fsub_rn(Y[a], __fmul_rn(e1, Wr[a]));
-    }
-    const float my = __fmul_rn(g, mag_y);
-    test(__fadd_rn(row_max32(sp, lo, hi), my), mag_y);
-    test(-__fsub_rn(row_min32(sm, lo, hi), my), mag_y);
-    // a test decided as culling settles it; otherwise every test must be decided
-    if (culled) return 1;
-    return undecided ? -1 : 0;
-}
+// What one view makes of one batch (or LOD node).
+struct BatchTest {
+    bool culled;   // outside the view for certain (Sec. 3.2)
+    bool front;    // every corner is in front of the eye; else the extents are unset
+    float fmin0, fmax0, fmin1, fmax1;   // spread of the corners' unfloored pixels
+    bool inside;   // the certificate of the raster kernels' fast path
+};
 
-__device__ __forceinline__ bool cull_batch(const pc_batch& b, const ViewParams& v) {
-    const int r = cull_batch_fast(b, v);
-    return r < 0 ? cull_batch_exact(b, v) : r == 1;
-}
-
-// Certificate of the raster kernel's fast path for one batch and view. True
-// only if, for every point the batch can decode to (all lie in
-// [min, fl(min + size)]), (1) the binary32 clip w lies in [2^-99, 2^99], so the
-// point is in front of the eye and the reciprocal estimate stays normal,
-// (2) c / w lies in [-1, 1 - 2^-20] on both axes, so the definition's floor
-// pixel is inside the view, and (3) every size is at most 2^100, so that the
-// decode constants 2^23 cell and 2^13 cell are exact. False is always safe: the
-// batch then takes the general path with per-point tests.
+// The three tests of a (batch, view) pair by a team of 8 lanes (l: the lane's
+// index in its team), so that the chain of dependent operations is one corner,
+// one plane and one quotient long; every lane of a team returns the result. All
+// 32 lanes of the warp must take part.
 //
-// Bounds in binary32: each row's exact range over the box, widened by 32u times
-// the magnitude of its terms (u = 2^-24). That covers the point's own rounding
-// (at most 6u of the magnitude, as for culling) plus the rounding of these
-// bounds (about 6u more), and 2^-120 covers underflow. The quotient bounds take
-// the interval endpoints (w > 0) and must clear the limits by 2^-12, far more
-// than the binary32 rounding of the bound itself.
-__device__ bool batch_fast(const pc_batch& b, const ViewParams& v) {
-    if (v.flags & PC_VIEW_NO_EARLY_DEPTH) return false;
+// Corners: lane l projects corner l with the same binary32 operations as a
+// point. A corner with w <= 0 clears `front`. As in a running minimum over the
+// corners in order, a NaN of corner 0 stays, a NaN of a later one is passed over.
+//
+// Culling, in binary32 first: lanes 0..4 take one clip plane each (w > 0, x >= -w,
+// x <= w, y >= -w, y <= w). Each test value t approximates the exact value R of
+// its expression within about 10 * 2^-24 of the magnitude M of its terms, and
+// the binary64 value within about 10 * 2^-53 M, so when |t| > 2^-16 M both have
+// the sign of R and the decision equals the binary64 one: culled when t < 0.
+// Inside that band, or when a magnitude is not finite or below 2^-90 (where
+// products could lose bits to underflow), the binary64 code decides.
+//
+// Certificate of the raster kernels' fast path: true only if, for every point
+// the batch can decode to (all lie in [min, fl(min + size)]), (1) the binary32
+// clip w lies in [2^-99, 2^99], so the point is in front of the eye and the
+// reciprocal estimate stays normal, (2) c / w lies in [-1, 1 - 2^-20] on both
+// axes, so the definition's floor pixel is inside the view, and (3) every size
+// is at most 2^100, so that the decode constants 2^23 cell and 2^13 cell are
+// exact. False is always safe: the batch then takes the general path with
+// per-point tests. Bounds in binary32: each row's exact range over the box,
+// widened by 32u times the magnitude of its terms (u = 2^-24). That covers the
+// point's own rounding (at most 6u of the magnitude, as for culling) plus the
+// rounding of these bounds (about 6u more), and 2^-120 covers underflow. The
+// quotient bounds take the interval endpoints (w > 0) and must clear the limits
+// by 2^-12, far more than the binary32 rounding of the bound itself. Lanes 1..4
+// take the lower and upper quotient of x and of y.
+__device__ __forceinline__ BatchTest test_batch(const pc_batch& b, const ViewParams& v, uint32_t l,
+                                                bool need_cull) {
+    const uint32_t team = 0xFFu << (threadIdx.x & 24u);   // this team's lanes in a ballot
+    const float* m = v.m;
     float lo[3], hi[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-        if (!(b.size[a] <= 0x1.0p100f)) return false;   // also NaN and infinities
         lo[a] = b.min[a];
         hi[a] = __fadd_rn(b.min[a], b.size[a]);
     }
-    const float* m = v.m;
-    const float X[4] = {m[0], m[4], m[8], m[12]};
-    const float Y[4] = {m[1], m[5], m[9], m[13]};
-    const float Wr[4] = {m[3], m[7], m[11], m[15]};
-    const float g = 32.0f * 0x1.0p-24f, tiny = 0x1.0p-120f;
-    const float mw = __fadd_rn(__fmul_rn(g, row_mag32(Wr, lo, hi)), tiny);
-    const float wl = __fsub_rn(row_min32(Wr, lo, hi), mw);
-    const float wh = __fadd_rn(row_max32(Wr, lo, hi), mw);
-    if (!(wl >= 0x1.0p-99f) || !(wh <= 0x1.0p99f)) return false;
-    const float lim_lo = -1.0f + 0x1.0p-12f, lim_hi = 1.0f - 0x1.0p-12f;
-    const float* rows[2] = {X, Y};
+    BatchTest r;
+    // corners
+    {
+        const float x = (l & 1u) ? hi[0] : lo[0], y = (l & 2u) ? hi[1] : lo[1];
+        const float z = (l & 4u) ? hi[2] : lo[2];
+        const float cw = clip_row(m, 3, x, y, z);
+        r.front = !(__ballot_sync(FULL, !(cw > 0.0f)) & team);
+        const float f0 = to_pixel(clip_row(m, 0, x, y, z), cw, (float)v.width);
+        const float f1 = to_pixel(clip_row(m, 1, x, y, z), cw, (float)v.height);
+        r.fmin0 = r.fmax0 = f0;
+        r.fmin1 = r.fmax1 = f1;
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-        const float mr = __fadd_rn(__fmul_rn(g, row_mag32(rows[r], lo, hi)), tiny);
-        const float cl = __fsub_rn(row_min32(rows[r], lo, hi), mr);
-        const float ch = __fadd_rn(row_max32(rows[r], lo, hi), mr);
-        const float qmin = cl >= 0.0f ? __fdiv_rn(cl, wh) : __fdiv_rn(cl, wl);
-        const float qmax = ch >= 0.0f ? __fdiv_rn(ch, wl) : __fdiv_rn(ch, wh);
-        if (!(qmin >= lim_lo) || !(qmax <= lim_hi)) return false;
+        for (int d = 1; d < 8; d <<= 1) {
+            r.fmin0 = fminf(r.fmin0, __shfl_xor_sync(FULL, r.fmin0, d));
+            r.fmax0 = fmaxf(r.fmax0, __shfl_xor_sync(FULL, r.fmax0, d));
+            r.fmin1 = fminf(r.fmin1, __shfl_xor_sync(FULL, r.fmin1, d));
+            r.fmax1 = fmaxf(r.fmax1, __shfl_xor_sync(FULL, r.fmax1, d));
+        }
+        const float first0 = __shfl_sync(FULL, f0, 0, 8), first1 = __shfl_sync(FULL, f1, 0, 8);
+        if (first0 != first0) r.fmin0 = r.fmax0 = first0;
+        if (first1 != first1) r.fmin1 = r.fmax1 = first1;
     }
-    return true;
+    // this lane's row: x for lanes 1 and 2, y for 3 and 4, w for lane 0
+    const float e1 = 1.0f + 0x1.0p-10f;
+    const float Wr[4] = {m[3], m[7], m[11], m[15]};
+    float R[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) R[a] = l <= 2u ? m[4 * a] : m[4 * a + 1];
+    const float bw = row_mag32(Wr, lo, hi), br = row_mag32(R, lo, hi);
+    r.culled = false;
+    if (need_cull) {
+        const float g = 6.0f * 0x1.0p-24f, band = 0x1.0p-16f;
+        const float mag = l == 0u ? bw : __fadd_rn(br, __fmul_rn(e1, bw));
+        float sp[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            sp[a] = l == 0u ? Wr[a] : __fadd_rn((l & 1u) ? R[a] : -R[a], __fmul_rn(e1, Wr[a]));
+        const float t = __fadd_rn(row_max32(sp, lo, hi), __fmul_rn(g, mag));
+        const float lim = __fmul_rn(band, mag);
+        const bool test = l <= 4u;
+        const bool range = !(bw <= 0x1.0p100f) || !(mag <= 0x1.0p100f) || !(bw >= 0x1.0p-90f) ||
+                           !(mag >= 0x1.0p-90f);
+        const bool bad = __ballot_sync(FULL, test && range) & team;
+        const bool out = __ballot_sync(FULL, test && t < -lim) & team;
+        const bool open = __ballot_sync(FULL, test && !(t < -lim) && !(t > lim)) & team;
+        // a plane decided as culling settles it; otherwise every plane must be decided
+        if (bad || (open && !out)) r.culled = cull_batch_exact(b, v);
+        else r.culled = out;
+    }
+    // certificate
+    {
+        const float g = 32.0f * 0x1.0p-24f, tiny = 0x1.0p-120f;
+        const float mw = __fadd_rn(__fmul_rn(g, bw), tiny);
+        const float wl = __fsub_rn(row_min32(Wr, lo, hi), mw);
+        const float wh = __fadd_rn(row_max32(Wr, lo, hi), mw);
+        const float mr = __fadd_rn(__fmul_rn(g, br), tiny);
+        const bool upper = !(l & 1u);
+        const float c = upper ? __fadd_rn(row_max32(R, lo, hi), mr) : __fsub_rn(row_min32(R, lo, hi), mr);
+        const float q = __fdiv_rn(c, (c >= 0.0f) == upper ? wl : wh);
+        const float lim = 1.0f - 0x1.0p-12f;
+        const bool ok = upper ? q <= lim : q >= -lim;
+        const bool fails = __ballot_sync(FULL, l >= 1u && l <= 4u && !ok) & team;
+        r.inside = !fails && !(v.flags & PC_VIEW_NO_EARLY_DEPTH) && wl >= 0x1.0p-99f &&
+                   wh <= 0x1.0p99f && b.size[0] <= 0x1.0p100f && b.size[1] <= 0x1.0p100f &&
+                   b.size[2] <= 0x1.0p100f;
+    }
+    return r;
 }
 
-constexpr int kCullThreads = 128;
-
-// Sum of a 64-bit value over the 32 lanes of a warp (butterfly on 32-bit
-// halves with the carry).
-__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
-    uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
-#pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) {
-        const uint32_t ol = __shfl_xor_sync(FULL, lo, d), oh = __shfl_xor_sync(FULL, hi, d);
-        const uint32_t nl = lo + ol;
-        hi = hi + oh + (nl < lo ? 1u : 0u);
-        lo = nl;
-    }
-    return ((unsigned long long)hi << 32) | lo;
+// Sec. 3.3: smallest k whose cells are below the threshold, from the extent
+// of the 8 projected box corners; 3 when a corner is not in front of the eye.
+__device__ __forceinline__ int select_k(const BatchTest& t, uint32_t flags, float T) {
+    const uint32_t fk = (flags & PC_VIEW_K_MASK) >> 4;
+    if (fk >= 1) return (int)fk;
+    if (!t.front) return 3;
+    const float ex = __fsub_rn(t.fmax0, t.fmin0), ey = __fsub_rn(t.fmax1, t.fmin1);
+    if (ex < T && ey < T) return 1;
+    const float T2 = __fmul_rn(T, 1024.0f);
+    if (ex < T2 && ey < T2) return 2;
+    return 3;
 }
 
 // Sec. 3.5: a node passes a view when it is in the frustum and, unless it is
 // the root, its projected extent reaches the view's threshold (a corner with
-// w <= 0 counts as large). lod_sel[n] gets one bit per view of the launch.
-__global__ void __launch_bounds__(kCullThreads) k_lod_pass(CloudView c, ViewTable vt, Scratch s) {
-    const uint32_t n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= c.n_batches) return;
-    const pc_batch bt = c.batches[n];
-    uint32_t mask = 0;
-    for (uint32_t v = 0; v < vt.n; ++v) {
-        const ViewParams& vp = vt.v[v];
-        if (cull_batch(bt, vp)) continue;
-        if (n > 0) {
-            float fmin0, fmax0, fmin1, fmax1;
-            if (corner_box(bt, vp, fmin0, fmax0, fmin1, fmax1)) {
-                const float ex = __fsub_rn(fmax0, fmin0), ey = __fsub_rn(fmax1, fmin1);
-                const float e = (ex != ex || ey != ey) ? __fadd_rn(ex, ey) : fmaxf(ex, ey);
-                float t = vp.lod_px;
-                if (vp.lod_px_periphery > 0.0f) {
-                    const float cx = __fmul_rn(__fadd_rn(fmin0, fmax0), 0.5f);
-                    const float cy = __fmul_rn(__fadd_rn(fmin1, fmax1), 0.5f);
-                    const int r = ring_of(cx, cy, vp.width, vp.height);
-                    if (r == 1) t = __fmul_rn(__fadd_rn(vp.lod_px, vp.lod_px_periphery), 0.5f);
-                    if (r == 2) t = vp.lod_px_periphery;
-                }
-                if (e < t) continue;
-            }
-        }
-        mask |= 1u << v;
+// w <= 0 counts as large).
+__device__ __forceinline__ bool lod_passes(const BatchTest& t, const ViewParams& vp, bool root) {
+    if (t.culled) return false;
+    if (root || !t.front) return true;
+    const float ex = __fsub_rn(t.fmax0, t.fmin0), ey = __fsub_rn(t.fmax1, t.fmin1);
+    const float e = (ex != ex || ey != ey) ? __fadd_rn(ex, ey) : fmaxf(ex, ey);
+    float limit = vp.lod_px;
+    if (vp.lod_px_periphery > 0.0f) {
+        const float cx = __fmul_rn(__fadd_rn(t.fmin0, t.fmax0), 0.5f);
+        const float cy = __fmul_rn(__fadd_rn(t.fmin1, t.fmax1), 0.5f);
+        const int r = ring_of(cx, cy, vp.width, vp.height);
+        if (r == 1) limit = __fmul_rn(__fadd_rn(vp.lod_px, vp.lod_px_periphery), 0.5f);
+        if (r == 2) limit = vp.lod_px_periphery;
     }
-    s.lod_sel[n] = mask;
+    return !(e < limit);
 }
 
-__global__ void __launch_bounds__(kCullThreads) k_cull(CloudView c, ViewTable vt, uint32_t view_base,
-                                                     Scratch s) {
-    __shared__ unsigned long long sh_stats[kMaxViewsPerLaunch * S_COUNT];
-    __shared__ unsigned long long sh_words;
-    for (uint32_t i = threadIdx.x; i < vt.n * S_COUNT; i += blockDim.x) sh_stats[i] = 0ull;
-    if (threadIdx.x == 0) sh_words = 0ull;
-    __syncthreads();
+// ---- draw list -----------------------------------------------------------------
 
-    const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-    uint32_t mask = 0, fmask = 0, nseg = 0, count = 0;
-    uint64_t kcodes = 0;
-    if (b < c.n_batches) {
-        const pc_batch bt = c.batches[b];
-        count = bt.count;
+// Blocks of the cull pass take up to kCullBatches batches each.
+constexpr uint32_t kCullThreads = 256, kCullTeams = kCullThreads / 8, kCullBatches = 128;
+
+// Exact sum of a 32-bit value over the warp's lanes, from two halves.
+__device__ __forceinline__ unsigned long long warp_sum(uint32_t v) {
+    return (unsigned long long)__reduce_add_sync(FULL, v & 0xFFFFu) +
+           ((unsigned long long)__reduce_add_sync(FULL, v >> 16) << 16);
+}
+
+// A block's batches and what they add to the draw list and the statistics.
+struct CullShared {
+    LodSel sel[kCullBatches];
+    uint32_t count[kCullBatches];
+    uint32_t nseg[kCullBatches];
+    unsigned long long pos[kCullBatches];
+    uint32_t batches[kMaxViewsPerLaunch][3];    // per view and k: batches, and their
+    uint32_t lo[kMaxViewsPerLaunch][3];         // points as sums of 16-bit halves
+    uint32_t hi[kMaxViewsPerLaunch][3];
+    unsigned long long words;
+};
+
+// Appends the block's n batches (sh.sel, sh.count; first: the first one's index)
+// to the draw list, in segments, and adds them to the statistics. One 64-bit
+// atomic per warp of batches reserves both parts of the list: entries from the
+// front, and, for one view, from the back those of batches not certified for the
+// fast path. Called by all threads after a __syncthreads().
+__device__ void append_batches(CullShared& sh, uint32_t first, uint32_t n, const ViewTable& vt,
+                               const Scratch& s) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (threadIdx.x < kCullBatches && (threadIdx.x & ~31u) < n) {
+        const uint32_t i = threadIdx.x;
+        uint32_t nseg = 0;
+        bool general = false;
+        uint32_t kl = 0;
+        if (i < n) {
+            const LodSel& e = sh.sel[i];
+            if (e.mask) nseg = (sh.count[i] + vt.seg_points - 1) / vt.seg_points;
+            general = vt.n == 1 && !(e.fast & 1u);
+            // the largest k of the drawn views: bit 1 set in any code of 2 or 3
+            // (codes of views that do not draw the batch are 0)
+            const uint64_t hi = e.kcodes & 0xAAAAAAAAAAAAAAAAull, lo = e.kcodes & 0x5555555555555555ull;
+            kl = !e.mask ? 0u : !hi ? 1u : (lo & (hi >> 1)) ? 3u : 2u;
+        }
+        unsigned long long incl = general ? (unsigned long long)nseg << 32 : nseg;
+        const unsigned long long own = incl;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned long long t = __shfl_up_sync(FULL, incl, d);
+            if (lane >= (uint32_t)d) incl += t;
+        }
+        const unsigned long long total = __shfl_sync(FULL, incl, 31);
+        unsigned long long base = 0;
+        if (lane == 31 && total)
+            base = atomicAdd(reinterpret_cast<unsigned long long*>(s.counters + C_ENTRIES), total);
+        const uint32_t count = i < n ? sh.count[i] : 0u;
+        const unsigned long long words = warp_sum(kl == 0u ? 0u : count) +
+                                         warp_sum(kl >= 2u ? count : 0u) + warp_sum(kl == 3u ? count : 0u);
+        if (lane == 0 && words) atomicAdd(&sh.words, words);
+        base = __shfl_sync(FULL, base, 31);
+        // both lists together fit the buffer up to this warp's reservation, or none
+        // of its entries is written (later reservations do not fit then either)
+        const uint64_t end = (base >> 32) + (uint32_t)base + (total >> 32) + (uint32_t)total;
+        if (end > s.capacity) {
+            if (nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)end);
+            nseg = 0;
+        }
+        if (i < n) {
+            const unsigned long long at = base + incl - own;
+            sh.nseg[i] = nseg;
+            sh.pos[i] = general ? s.capacity - 1u - (at >> 32) : (uint32_t)at;
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x >> 3; i < n; i += kCullTeams) {
+        const LodSel sel = sh.sel[i];
+        const bool general = vt.n == 1 && !(sel.fast & 1u);
+        const uint32_t count = sh.count[i], nseg = sh.nseg[i];
+        for (uint32_t g = threadIdx.x & 7u; g < nseg; g += 8u) {
+            DrawEntry e;
+            e.kcodes = sel.kcodes;
+            e.view_mask = sel.mask;
+            e.fast_mask = sel.fast;
+            e.pad = 0;
+            e.batch = first + i;
+            e.seg_first = g * vt.seg_points;
+            e.seg_count = min(vt.seg_points, count - g * vt.seg_points);
+            s.entries[general ? sh.pos[i] - g : sh.pos[i] + g] = e;
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < vt.n * 3u; i += blockDim.x) {
+        const uint32_t v = i / 3u, k = i % 3u, nb = sh.batches[v][k];
+        if (!nb) continue;
+        unsigned long long* st = s.acc + (uint64_t)v * S_COUNT;
+        atomicAdd(st + S_BATCHES, (unsigned long long)nb);
+        atomicAdd(st + S_BK1 + k, (unsigned long long)nb);
+        atomicAdd(st + S_PK1 + k, (unsigned long long)sh.lo[v][k] + ((unsigned long long)sh.hi[v][k] << 16));
+    }
+    // the whole launch group's word loads, for each of its views
+    if (threadIdx.x < vt.n && sh.words)
+        atomicAdd(s.acc + (uint64_t)threadIdx.x * S_COUNT + S_WORDS, sh.words);
+}
+
+// A drawn batch of one view at precision k, for the block's statistics.
+__device__ __forceinline__ void count_batch(CullShared& sh, uint32_t v, uint32_t k, uint32_t count) {
+    atomicAdd(&sh.batches[v][k - 1], 1u);
+    atomicAdd(&sh.lo[v][k - 1], count & 0xFFFFu);
+    atomicAdd(&sh.hi[v][k - 1], count >> 16);
+}
+
+__device__ __forceinline__ void init_cull(CullShared& sh, uint32_t nviews) {
+    for (uint32_t i = threadIdx.x; i < nviews * 3u; i += blockDim.x)
+        sh.batches[i / 3u][i % 3u] = sh.lo[i / 3u][i % 3u] = sh.hi[i / 3u][i % 3u] = 0u;
+    if (threadIdx.x < kCullBatches) {
+        sh.sel[threadIdx.x].kcodes = 0ull;
+        sh.sel[threadIdx.x].mask = sh.sel[threadIdx.x].fast = 0u;
+    }
+    if (threadIdx.x == 0) sh.words = 0ull;
+}
+
+// The first pass of a frame: blocks [0, cull_blocks) test every batch against
+// every view, a team of 8 lanes per pair; the others clear the views' buffers,
+// which nothing needs before the next kernel. A plain cloud's batches go to the
+// draw list at once, an LOD cloud's nodes only note their results (a node is drawn
+// when its ancestors pass too: k_lod_append).
+// Bound by latency: the batch's load, the tests' chain and one atomic. One thread
+// per batch, with the views in turn, and a clear pass before it took 19 us for a
+// 1M-point cloud at 512x512 (65 us with 16 views, 43 us for 2B points at 1080p);
+// this pass takes 11 us (25 and 39 us). Four blocks per SM (64 registers): with
+// the 89 registers it would take, the 2B frame's 195,313 batches need 53 us.
+__global__ void __launch_bounds__(kCullThreads, 4) k_begin(CloudView c, ViewTable vt, Scratch s,
+                                                      uint32_t cull_blocks, uint32_t per_block,
+                                                      uint32_t clear_parts) {
+    if (blockIdx.x >= cull_blocks) {
+        const uint32_t j = blockIdx.x - cull_blocks;
+        clear_view(vt.v[j / clear_parts], j % clear_parts, clear_parts);
+        return;
+    }
+    __shared__ CullShared sh;
+    init_cull(sh, vt.n);
+    __syncthreads();
+    const uint32_t first = blockIdx.x * per_block, n = min(per_block, c.n_batches - first);
+    const uint32_t l = threadIdx.x & 7u, items = n * vt.n;
+    for (uint32_t i0 = 0; i0 < items; i0 += kCullTeams) {
+        const uint32_t item = i0 + (threadIdx.x >> 3);
+        const bool active = item < items;
+        // views in the outer order: a warp's teams mostly share their view
+        const uint32_t v = active ? item / n : 0u, i = active ? item % n : 0u;
+        const pc_batch bt = c.batches[first + i];
+        const ViewParams& vp = vt.v[v];
+        const BatchTest t = test_batch(bt, vp, l, c.is_lod || (vp.flags & PC_VIEW_CULL));
+        if (!active || l != 0u) continue;
+        uint32_t count = bt.count;
         if ((uint64_t)bt.first + bt.count > c.n_points) {
-            raise_error(s, E_BATCH_RANGE, b);
+            raise_error(s, E_BATCH_RANGE, first + i);
             count = 0;
         }
-        uint32_t lod_mask = ~0u;
-        if (c.is_lod) {
-            // drawn when this node and every ancestor passed (parents come
-            // first in breadth-first order; the root is its own parent)
-            lod_mask = s.lod_sel[b];
-            uint32_t node = b;
-            for (int depth = 0; depth < 64 && lod_mask; ++depth) {
-                const uint32_t par = c.parent[node];
-                if (par == node || par >= c.n_batches) break;
-                lod_mask &= s.lod_sel[par];
-                node = par;
-            }
-        }
-        for (uint32_t v = 0; v < vt.n && count; ++v) {
-            const ViewParams& vp = vt.v[v];
-            if (c.is_lod) {
-                if (!((lod_mask >> v) & 1u)) continue;
-            } else if ((vp.flags & PC_VIEW_CULL) && cull_batch(bt, vp)) {
-                continue;
-            }
-            const int k = select_k(bt, vp, vt.threshold_px);
-            mask |= 1u << v;
-            kcodes |= (uint64_t)k << (2 * v);
-            if (k <= 2 && batch_fast(bt, vp)) fmask |= 1u << v;
-        }
-        if (mask) nseg = (count + vt.seg_points - 1) / vt.seg_points;
-    }
-    const uint32_t lane = threadIdx.x & 31;
-    // statistics, summed over the warp first: one shared-memory addition per
-    // warp and counter (64-bit shared atomics contend badly lane by lane)
-    uint32_t kl = 0;
-    for (uint32_t v = 0; v < vt.n; ++v) {
-        const bool drawn = (mask >> v) & 1u;
-        if (!__any_sync(FULL, drawn)) continue;
-        const uint32_t k = (uint32_t)((kcodes >> (2 * v)) & 3u);
-        if (drawn) kl = max(kl, k);
-        uint32_t nb = 0;
-#pragma unroll
-        for (uint32_t kk = 1; kk <= 3; ++kk) {
-            const bool sel = drawn && k == kk;
-            const uint32_t n = __popc(__ballot_sync(FULL, sel));
-            const unsigned long long pts = warp_sum_u64(sel ? count : 0u);
-            nb += n;
-            if (lane == 0 && n) {
-                atomicAdd(&sh_stats[v * S_COUNT + S_BK1 + (kk - 1)], (unsigned long long)n);
-                atomicAdd(&sh_stats[v * S_COUNT + S_PK1 + (kk - 1)], pts);
-            }
-        }
-        if (lane == 0) atomicAdd(&sh_stats[v * S_COUNT + S_BATCHES], (unsigned long long)nb);
-    }
-    {
-        const unsigned long long words = warp_sum_u64((unsigned long long)kl * (mask ? count : 0u));
-        if (lane == 0 && words) atomicAdd(&sh_words, words);
-    }
-    // warp-aggregated append of nseg entries: the front list, and for one view
-    // the list from the back for batches without the fast path
-    const bool general = vt.n == 1 && !(fmask & 1u);
-    unsigned long long incl = general ? (unsigned long long)nseg << 32 : nseg;
-    const unsigned long long own = incl;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long t = __shfl_up_sync(FULL, incl, d);
-        if (lane >= (uint32_t)d) incl += t;
-    }
-    const unsigned long long total = __shfl_sync(FULL, incl, 31);
-    unsigned long long base = 0;
-    if (lane == 31 && total)
-        base = atomicAdd(reinterpret_cast<unsigned long long*>(s.counters + C_ENTRIES), total);
-    base = __shfl_sync(FULL, base, 31);
-    // both lists together fit the buffer up to this warp's reservation, or none
-    // of its entries is written (later reservations do not fit then either)
-    const uint64_t end = (base >> 32) + (uint32_t)base + (total >> 32) + (uint32_t)total;
-    if (end > s.capacity) {
-        if (nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)end);
-        nseg = 0;
-    }
-    const unsigned long long at = base + incl - own;
-    uint64_t pos = general ? s.capacity - 1u - (at >> 32) : (uint32_t)at;
-    for (uint32_t g = 0; g < nseg; ++g, pos += general ? -1ll : 1ll) {
-        DrawEntry e;
-        e.kcodes = kcodes;
-        e.view_mask = mask;
-        e.fast_mask = fmask;
-        e.pad = 0;
-        e.batch = b;
-        e.seg_first = g * vt.seg_points;
-        e.seg_count = min(vt.seg_points, count - g * vt.seg_points);
-        s.entries[pos] = e;
+        if (v == 0) sh.count[i] = count;
+        const bool drawn = c.is_lod ? lod_passes(t, vp, first + i == 0) : !t.culled;
+        // a plain batch without points is not drawn; a node's children may be
+        if (!drawn || (!count && !c.is_lod)) continue;
+        const int k = select_k(t, vp.flags, vt.threshold_px);
+        atomicOr(&sh.sel[i].mask, 1u << v);
+        atomicOr(&sh.sel[i].kcodes, (unsigned long long)k << (2u * v));
+        if (k <= 2 && t.inside) atomicOr(&sh.sel[i].fast, 1u << v);
+        if (!c.is_lod) count_batch(sh, v, (uint32_t)k, count);
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < vt.n * S_COUNT; i += blockDim.x) {
-        unsigned long long x = sh_stats[i];
-        if (i % S_COUNT == S_WORDS) x = sh_words;   // the whole launch group's word loads
-        if (x && i % S_COUNT <= S_WORDS) atomicAdd(&s.stats[(uint64_t)view_base * S_COUNT + i], x);
+    if (c.is_lod) {
+        for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s.lod_sel[first + i] = sh.sel[i];
+        return;
     }
+    append_batches(sh, first, n, vt, s);
+}
+
+// LOD clouds: the nodes that pass some view together with all their ancestors
+// (parents come first in breadth-first order; the root is its own parent).
+__global__ void __launch_bounds__(kCullThreads) k_lod_append(CloudView c, ViewTable vt, Scratch s,
+                                                           uint32_t per_block) {
+    __shared__ CullShared sh;
+    init_cull(sh, vt.n);
+    __syncthreads();
+    const uint32_t first = blockIdx.x * per_block, n = min(per_block, c.n_batches - first);
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        LodSel e = s.lod_sel[first + i];
+        uint32_t node = first + i, mask = e.mask;
+        for (int depth = 0; depth < 64 && mask; ++depth) {
+            const uint32_t par = c.parent[node];
+            if (par == node || par >= c.n_batches) break;
+            mask &= s.lod_sel[par].mask;
+            node = par;
+        }
+        if (!mask) continue;
+        const pc_batch bt = c.batches[first + i];
+        uint32_t count = bt.count;
+        if ((uint64_t)bt.first + bt.count > c.n_points) count = 0;   // reported by k_begin
+        sh.count[i] = count;
+        if (!count) continue;
+        uint64_t codes = 0;
+        for (uint32_t m = mask; m; m &= m - 1) {
+            const uint32_t v = __ffs(m) - 1, k = (uint32_t)(e.kcodes >> (2u * v)) & 3u;
+            codes |= (uint64_t)k << (2u * v);
+            count_batch(sh, v, k, count);
+        }
+        sh.sel[i].mask = mask;
+        sh.sel[i].fast = e.fast & mask;
+        sh.sel[i].kcodes = codes;
+    }
+    __syncthreads();
+    append_batches(sh, first, n, vt, s);
 }
 
 // Hardware reciprocal approximation; used only for w in [2^-100, 2^100], where
@@ -1321,7 +1355,7 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
                                               uint32_t lane) {
     const uint32_t t = __reduce_add_sync(FULL, n_atom);
     if (lane == 0 && t)
-        atomicAdd(&s.stats[(uint64_t)view * S_COUNT + S_ATOMICS], (unsigned long long)t);
+        atomicAdd(&s.acc[(uint64_t)view * S_COUNT + S_ATOMICS], (unsigned long long)t);
 }
 
 // One view per launch: two kernels, so that neither path's registers burden the
@@ -1337,7 +1371,7 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
 // Five blocks of 256 threads per SM (48 registers): the depth reads' latency is
 // hidden by other warps, and more warps hide more of it.
 __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c, ViewTable vt,
-                                                               uint32_t view_base, Scratch s) {
+                                                               Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
@@ -1354,13 +1388,13 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c, 
         n_atom += (e.kcodes & 3u) == 1u ? segment_fast<1, true>(c, fv, bt, p0, p1, lane)
                                         : segment_fast<2, true>(c, fv, bt, p0, p1, lane);
     }
-    flush_atomics(s, view_base, n_atom, lane);
+    flush_atomics(s, 0u, n_atom, lane);
     // what follows in the stream waits for this kernel: it ends after the other
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView c, ViewTable vt,
-                                                                  uint32_t view_base, Scratch s) {
+                                                                  Scratch s) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_front, n_entries;
@@ -1378,14 +1412,14 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView 
         const uint32_t p0 = bt.first + e.seg_first;
         n_atom += segment_k<true>(c, vc, bt, (int)(e.kcodes & 3u), p0, p0 + e.seg_count, lane);
     }
-    flush_atomics(s, view_base, n_atom, lane);
+    flush_atomics(s, 0u, n_atom, lane);
 }
 
 // Two views per launch (a stereo pair, Sec. 3.7): as k_rasterN, with both
 // views' constants at fixed parameter offsets. Four blocks of 256 threads per
 // SM (64 registers).
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, ViewTable vt,
-                                                           uint32_t view_base, Scratch s) {
+                                                           Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
@@ -1417,8 +1451,8 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, View
             na1 += segment_k<false>(c, make_view_const(vt.v[1]), bt, (int)((e.kcodes >> 2) & 3u),
                                     p0, p1, lane);
     }
-    flush_atomics(s, view_base, na0, lane);
-    flush_atomics(s, view_base + 1, na1, lane);
+    flush_atomics(s, 0u, na0, lane);
+    flush_atomics(s, 1u, na1, lane);
 }
 
 // Several views per launch (Sec. 3.7): the views certified for a segment's
@@ -1427,7 +1461,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, View
 // view keeps its own culling and precision, so each image is the one-view
 // image bit for bit.
 __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, ViewTable vt,
-                                                           uint32_t view_base, Scratch s) {
+                                                           Scratch s) {
     __shared__ uint32_t sh_atom[kMaxViewsPerLaunch];
     for (uint32_t i = threadIdx.x; i < kMaxViewsPerLaunch; i += blockDim.x) sh_atom[i] = 0;
     __syncthreads();
@@ -1464,8 +1498,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, View
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < vt.n; i += blockDim.x)
         if (sh_atom[i])
-            atomicAdd(&s.stats[(uint64_t)(view_base + i) * S_COUNT + S_ATOMICS],
-                      (unsigned long long)sh_atom[i]);
+            atomicAdd(&s.acc[(uint64_t)i * S_COUNT + S_ATOMICS], (unsigned long long)sh_atom[i]);
 }
 
 // ---- k_shade: Sec. 3.6 high-quality shading, colour pass ---------------------------
@@ -1818,7 +1851,7 @@ __device__ __forceinline__ uint32_t shade_segment_k(const CloudView& c, const Vi
 // Four blocks of 256 threads per SM (64 registers): the kernel waits on loads
 // and on the visibility reads at run starts, and more warps hide more of it.
 template <int LAYOUTS, bool ONE>
-__global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, uint32_t view_base, Scratch s,
+__global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, Scratch s,
                         uint32_t shade_mask) {
     constexpr bool FALLBACK = LAYOUTS == 0;
     __shared__ uint32_t sh_blend[kMaxViewsPerLaunch];
@@ -1826,7 +1859,7 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, uin
         uint32_t fb = 0;
         for (uint32_t mm = shade_mask; mm; mm &= mm - 1) {
             const uint32_t v = __ffs(mm) - 1;
-            if (s.stats[(uint64_t)(view_base + v) * S_COUNT + S_FALLBACK]) fb |= 1u << v;
+            if (s.acc[(uint64_t)v * S_COUNT + S_FALLBACK]) fb |= 1u << v;
         }
         if (!fb) return;
         shade_mask = fb;
@@ -1859,7 +1892,7 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, uin
             sb.sums = vp.accum;
             sb.flags = vp.accum + npix;
             sb.fallback = vp.accum + hqs_fallback_offset(npix);
-            sb.fallback_pixels = &s.stats[(uint64_t)(view_base + v) * S_COUNT + S_FALLBACK];
+            sb.fallback_pixels = &s.acc[(uint64_t)v * S_COUNT + S_FALLBACK];
             uint32_t n;
             if (FALLBACK)
                 n = shade_segment_k<ShadeMode::kFallback>(c, vc, fv, sb, bt, k, fast, p0,
@@ -1877,15 +1910,26 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, uin
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < vt.n; i += blockDim.x)
         if (sh_blend[i])
-            atomicAdd(&s.stats[(uint64_t)(view_base + i) * S_COUNT + S_BLENDED],
-                      (unsigned long long)sh_blend[i]);
+            atomicAdd(&s.acc[(uint64_t)i * S_COUNT + S_BLENDED], (unsigned long long)sh_blend[i]);
 }
 
 // ---- k_resolve ---------------------------------------------------------------------
 
-__global__ void k_resolve(CloudView c, ViewTable vt, Scratch s) {
+// The frame's last pass. With publish, its first block also hands the frame's
+// statistics over (stats of the launch's views from view_base on) and leaves the
+// accumulators and the draw-list counters at zero for the next frame, whose first
+// pass then needs no pass before it.
+__global__ void k_resolve(CloudView c, ViewTable vt, uint32_t view_base, Scratch s, bool publish) {
     const uint32_t v = blockIdx.y;
     if (v >= vt.n) return;
+    if (publish && v == 0 && blockIdx.x == 0) {
+        for (uint32_t i = threadIdx.x; i < vt.n * S_COUNT; i += blockDim.x) {
+            s.stats[(uint64_t)view_base * S_COUNT + i] = s.acc[i];
+            s.acc[i] = 0ull;
+        }
+        if (threadIdx.x < C_COUNT && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
+            s.counters[threadIdx.x] = 0u;
+    }
     const ViewParams& vp = vt.v[v];
     if (!vp.rgba) return;
     const uint64_t npix = (uint64_t)vp.width * vp.height;
@@ -2014,30 +2058,32 @@ int num_sms() {
 
 }  // namespace
 
-cudaError_t launch_clear(const ViewTable& vt, uint32_t view_base, Scratch s, cudaStream_t st) {
+// Batches per block of the cull pass: one round of its teams (fewer batches for
+// more views, so that a small cloud still spreads over the SMs), more when the
+// cloud has enough batches for four blocks per SM all the same (fewer blocks add
+// to the statistics).
+static uint32_t cull_batches_per_block(uint32_t n_batches, uint32_t nviews) {
+    const uint32_t round = std::max(1u, kCullTeams / std::max(1u, nviews));
+    const uint32_t spread = n_batches / ((uint32_t)num_sms() * 4u);
+    return std::min(kCullBatches, std::max(round, spread));
+}
+
+cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
     uint64_t maxpix = 0;
     for (uint32_t v = 0; v < vt.n; ++v)
         maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
-    const int threads = 256;
-    uint64_t blocks = (maxpix / 2 + threads - 1) / threads;
-    blocks = blocks < 1 ? 1 : (blocks > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : blocks);
-    dim3 grid((unsigned)blocks, vt.n ? vt.n : 1);
-    k_clear<<<grid, threads, 0, st>>>(vt, view_base, s);
+    uint64_t parts = (maxpix / 2 + kCullThreads - 1) / kCullThreads;
+    parts = parts < 1 ? 1 : (parts > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : parts);
+    const uint32_t per = cull_batches_per_block(c.n_batches, vt.n);
+    const uint32_t cull = (c.n_batches + per - 1) / per;
+    k_begin<<<cull + (uint32_t)parts * vt.n, kCullThreads, 0, st>>>(c, vt, s, cull, per, (uint32_t)parts);
     return cudaGetLastError();
 }
 
-cudaError_t launch_lod_pass(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
-    const unsigned blocks = (c.n_batches + kCullThreads - 1) / kCullThreads;
-    if (blocks == 0) return cudaSuccess;
-    k_lod_pass<<<blocks, kCullThreads, 0, st>>>(c, vt, s);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_cull(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
-                        cudaStream_t st) {
-    const unsigned blocks = (c.n_batches + kCullThreads - 1) / kCullThreads;
-    if (blocks == 0) return cudaSuccess;
-    k_cull<<<blocks, kCullThreads, 0, st>>>(c, vt, view_base, s);
+cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
+    if (c.n_batches == 0) return cudaSuccess;
+    const uint32_t per = cull_batches_per_block(c.n_batches, 1);
+    k_lod_append<<<(c.n_batches + per - 1) / per, kCullThreads, 0, st>>>(c, vt, s, per);
     return cudaGetLastError();
 }
 
@@ -2051,16 +2097,16 @@ int raster_occupancy(int threads_per_block, uint32_t nviews) {
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
+cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
                           RasterShape shape, cudaStream_t st, int* launched) {
     int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
     threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
     const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
     *launched = vt.n == 1 ? 2 : 1;
-    if (vt.n > 2) k_rasterN<<<blocks, threads, 0, st>>>(c, vt, view_base, s);
-    else if (vt.n == 2) k_raster2<<<blocks, threads, 0, st>>>(c, vt, view_base, s);
+    if (vt.n > 2) k_rasterN<<<blocks, threads, 0, st>>>(c, vt, s);
+    else if (vt.n == 2) k_raster2<<<blocks, threads, 0, st>>>(c, vt, s);
     if (vt.n != 1) return cudaGetLastError();
-    k_raster_general<<<num_sms() * 4, kRasterThreads, 0, st>>>(c, vt, view_base, s);
+    k_raster_general<<<num_sms() * 4, kRasterThreads, 0, st>>>(c, vt, s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute early{};
@@ -2072,28 +2118,28 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, uint32_t view
     cfg.stream = st;
     cfg.attrs = &early;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, vt, view_base, s);
+    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, vt, s);
 }
 
 template <int LAYOUTS>
-static cudaError_t launch_shade_kernel(const CloudView& c, const ViewTable& vt, uint32_t view_base,
+static cudaError_t launch_shade_kernel(const CloudView& c, const ViewTable& vt,
                                        Scratch s, int threads, uint32_t mask, cudaStream_t st) {
     int nb = 0;
     if constexpr (LAYOUTS != 3) {   // one view: the kernel with its index fixed
         if (vt.n == 1) {
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_shade<LAYOUTS, true>, threads, 0);
             const int blocks = num_sms() * (nb > 0 ? nb : 1);
-            k_shade<LAYOUTS, true><<<blocks, threads, 0, st>>>(c, vt, view_base, s, mask);
+            k_shade<LAYOUTS, true><<<blocks, threads, 0, st>>>(c, vt, s, mask);
             return cudaGetLastError();
         }
     }
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_shade<LAYOUTS, false>, threads, 0);
     const int blocks = num_sms() * (nb > 0 ? nb : 1);
-    k_shade<LAYOUTS, false><<<blocks, threads, 0, st>>>(c, vt, view_base, s, mask);
+    k_shade<LAYOUTS, false><<<blocks, threads, 0, st>>>(c, vt, s, mask);
     return cudaGetLastError();
 }
 
-cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
+cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, Scratch s,
                          RasterShape shape, cudaStream_t st, int* launched) {
     uint32_t mask = 0, packed = 0;
     for (uint32_t v = 0; v < vt.n; ++v) {
@@ -2106,12 +2152,12 @@ cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, uint32_t view_
     int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
     threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
     const int layouts = (mask != packed ? 1 : 0) | (packed ? 2 : 0);
-    cudaError_t e = layouts == 1 ? launch_shade_kernel<1>(c, vt, view_base, s, threads, mask, st)
-                  : layouts == 2 ? launch_shade_kernel<2>(c, vt, view_base, s, threads, mask, st)
-                                 : launch_shade_kernel<3>(c, vt, view_base, s, threads, mask, st);
+    cudaError_t e = layouts == 1 ? launch_shade_kernel<1>(c, vt, s, threads, mask, st)
+                  : layouts == 2 ? launch_shade_kernel<2>(c, vt, s, threads, mask, st)
+                                 : launch_shade_kernel<3>(c, vt, s, threads, mask, st);
     *launched = 1;
     if (e != cudaSuccess || !packed) return e;
-    e = launch_shade_kernel<0>(c, vt, view_base, s, threads, packed, st);
+    e = launch_shade_kernel<0>(c, vt, s, threads, packed, st);
     *launched = 2;
     return e;
 }
@@ -2126,7 +2172,8 @@ cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cud
     return cudaGetLastError();
 }
 
-cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
+cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
+                           bool publish, cudaStream_t st) {
     uint64_t maxpix = 0;
     for (uint32_t v = 0; v < vt.n; ++v)
         maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
@@ -2134,7 +2181,7 @@ cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, Scratch s, c
     uint64_t blocks = (maxpix + threads - 1) / threads;
     blocks = blocks < 1 ? 1 : (blocks > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : blocks);
     dim3 grid((unsigned)blocks, vt.n ? vt.n : 1);
-    k_resolve<<<grid, threads, 0, st>>>(c, vt, s);
+    k_resolve<<<grid, threads, 0, st>>>(c, vt, view_base, s, publish);
     return cudaGetLastError();
 }
 

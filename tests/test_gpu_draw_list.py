@@ -48,3 +48,45 @@ def test_mixed_lists_match_oracle(cuda_lib, n, batch, graphs):
             gst = ctx.stats(stream=stream)
             assert gst["batches_k"] == st["batches_k"]
             assert gst["points_atomic"] >= (ovis != O.EMPTY).sum()
+
+
+@pytest.mark.parametrize("nviews", [1, 2, 3, 5, 31, 32])
+@pytest.mark.parametrize("n,batch", [(3, 4), (31 * 8 + 5, 8), (33 * 8, 8), (1029, 8), (130_001, 64)])
+def test_cull_blocks_match_oracle(cuda_lib, n, batch, nviews):
+    """Counts of batches and views around the cull pass's blocks and rounds:
+    every view's image and counters are the oracle's."""
+    import torch
+    p = S.terrain_params(2000.0, 0.2, 30)
+    xyz, rgba = S.terrain(n, p, seed=6)
+    enc = O.encode(xyz, rgba, batch)
+    with pcr.Context(0, batch_size=batch) as ctx:
+        cloud = ctx.upload(xyz, rgba)
+        ms = [S.random_view(p, i, 40 + i, 33, seed=6) if i % 3 else S.overview(p, 40 + i, 33)
+              for i in range(nviews)]
+        views = [pcr.make_view(m, 40 + i, 33, pcr.PC_VIEW_CULL) for i, m in enumerate(ms)]
+        fbs = ctx.render(cloud, views)
+        torch.cuda.synchronize()
+        for i in range(0, nviews, 5):
+            ovis, st = O.render(enc, O.make_view(ms[i], 40 + i, 33, cull=True))
+            assert np.array_equal(pcr.vis_to_numpy(fbs[i][0]), ovis)
+            gst = ctx.stats(i)
+            assert gst["batches_k"] == st["batches_k"]
+            assert gst["points_k"] == st["points_k"]
+
+
+def test_statistics_survive_a_separate_resolve(cuda_lib):
+    """pc_resolve draws nothing, so the last frame's counters stay; the next
+    frame's start from zero."""
+    import torch
+    p = S.terrain_params(2000.0)
+    xyz, rgba = S.terrain(50_000, p, seed=7)
+    with pcr.Context(0) as ctx:
+        cloud = ctx.upload(xyz, rgba)
+        v = pcr.make_view(S.overview(p, 80, 50), 80, 50, pcr.PC_VIEW_CULL)
+        fbs = ctx.render(cloud, [v])
+        st = ctx.stats()
+        ctx.resolve(cloud, [v], fbs)
+        assert ctx.stats() == st and st["points_processed"] == 50_000
+        ctx.render(cloud, [v], fbs)
+        torch.cuda.synchronize()
+        assert ctx.stats()["points_k"] == st["points_k"]
