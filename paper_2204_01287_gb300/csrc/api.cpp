@@ -263,10 +263,11 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         cudaError_t e = cudaSuccess;
         if (fo.resolve_only) {
             if (fe) for (int i = 1; i < 5; ++i) cudaEventRecord(fe->ev[i], st);
-            e = launch_resolve(cv, vt, base, slot->scratch, false, st);
+            int resolve_kernels = 0;
+            e = launch_resolve(cv, vt, base, slot->scratch, false, st, &resolve_kernels);
             if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
             if (fe) cudaEventRecord(fe->ev[5], st);
-            launches += 1;
+            launches += resolve_kernels;
             continue;
         }
         if (fe) cudaEventRecord(fe->ev[1], st);   // the clear runs beside the culling
@@ -289,10 +290,11 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
             launches += nk;
         }
         if (fe) cudaEventRecord(fe->ev[4], st);
-        e = launch_resolve(cv, vt, base, slot->scratch, true, st);
+        int resolve_kernels = 0;
+        e = launch_resolve(cv, vt, base, slot->scratch, true, st, &resolve_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
         if (fe) cudaEventRecord(fe->ev[5], st);
-        launches += 2 + raster_kernels;
+        launches += 1 + raster_kernels + resolve_kernels;
         raster_launches += 1;
     }
     return PC_OK;

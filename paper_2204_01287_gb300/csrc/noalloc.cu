@@ -139,7 +139,7 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     int launched = 0;
     if (nbatches && launch_raster(c, vt, s, shape, st, &launched) != cudaSuccess)
         return PC_ECUDA;
-    if (launch_resolve(c, vt, 0, s, true, st) != cudaSuccess) return PC_ECUDA;
+    if (launch_resolve(c, vt, 0, s, true, st, &launched) != cudaSuccess) return PC_ECUDA;
     // the device error flag and its value, for the caller to read once the
     // stream has reached this point (a copy into caller memory, no allocation)
     if (device_error && cudaMemcpyAsync(device_error, L->counters + C_ERROR, 2 * sizeof(uint32_t),

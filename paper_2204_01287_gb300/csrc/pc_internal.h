@@ -178,7 +178,7 @@ cudaError_t launch_shade(const CloudView& c, const ViewTable& vt, Scratch s,
 // publish: the launch's statistics become stats[view_base ..] and the scratch
 // counters return to zero (every launch but a resolve alone).
 cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
-                           bool publish, cudaStream_t st);
+                           bool publish, cudaStream_t st, int* launched);
 // dst[i] = min(dst[i], src[i]) over n keys (both 16-byte aligned).
 cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cudaStream_t st);
 

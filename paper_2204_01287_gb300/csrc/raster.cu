@@ -1915,28 +1915,80 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, Scr
 
 // ---- k_resolve ---------------------------------------------------------------------
 
-// The frame's last pass. With publish, its first block also hands the frame's
+// What the frame's last pass does besides: its first block hands the frame's
 // statistics over (stats of the launch's views from view_base on) and leaves the
 // accumulators and the draw-list counters at zero for the next frame, whose first
 // pass then needs no pass before it.
+__device__ __forceinline__ void publish_frame(uint32_t nviews, uint32_t view_base, const Scratch& s) {
+    for (uint32_t i = threadIdx.x; i < nviews * S_COUNT; i += blockDim.x) {
+        s.stats[(uint64_t)view_base * S_COUNT + i] = s.acc[i];
+        s.acc[i] = 0ull;
+    }
+    if (threadIdx.x < C_COUNT && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
+        s.counters[threadIdx.x] = 0u;
+}
+
+// sum / n for a sum of n bytes (0 < n, sum <= 255 n < 2^32), rounded down: the
+// binary32 estimate is off by less than 2^-10, so its whole part is at most one off,
+// which the remainder corrects.
+__device__ __forceinline__ uint32_t average(uint32_t sum, uint32_t n, float inv) {
+    uint32_t q = (uint32_t)(__uint2float_rn(sum) * inv);
+    const uint32_t rem = sum - q * n;   // in (-n, 2n), modulo 2^32
+    if ((int32_t)rem < 0 && rem >= 0u - n) --q;
+    else if (rem >= n) ++q;
+    return q;
+}
+
+// The colour of a pixel that shows the point of `key`, whose own pixel is `at`:
+// the point's, or with shading (mode: hqs_mode) the average of that pixel's sums,
+// per channel and rounded down (Sec. 3.6).
+__device__ __forceinline__ uint32_t pixel_colour(const CloudView& c, const ViewParams& vp,
+                                                 uint64_t npix, uint32_t mode, unsigned long long key,
+                                                 uint64_t at, unsigned long long empty,
+                                                 const Scratch& s) {
+    if (key == empty) return 0u;
+    if (!mode) {
+        const uint32_t idx = (uint32_t)key;
+        if (idx < c.n_points) return c.color[idx];
+        raise_error(s, E_INDEX_RANGE, idx);
+        return 0u;
+    }
+    uint32_t r, g, b, n;
+    const ulonglong2* two = reinterpret_cast<const ulonglong2*>(vp.accum);   // two-word sums
+    bool use_two = mode == 1;
+    if (mode == 2) {
+        use_two = (vp.accum[npix + (at >> 6)] >> (at & 63)) & 1ull;
+        two = reinterpret_cast<const ulonglong2*>(vp.accum + hqs_fallback_offset(npix));
+        const unsigned long long a = vp.accum[at];
+        r = (uint32_t)(a & 0x3FFFFu);
+        g = (uint32_t)((a >> 18) & 0x3FFFFu);
+        b = (uint32_t)((a >> 36) & 0x3FFFFu);
+        n = (uint32_t)(a >> 54);
+    }
+    if (use_two) {
+        const ulonglong2 t = two[at];
+        r = (uint32_t)t.x;
+        g = (uint32_t)(t.x >> 32);
+        b = (uint32_t)t.y;
+        n = (uint32_t)(t.y >> 32);
+        if (n > kHqsMaxCount) raise_error(s, E_HQS_OVERFLOW, (uint32_t)at);
+    }
+    if (!n) return 0u;
+    const float inv = rcp_approx((float)n);
+    return average(r, n, inv) | (average(g, n, inv) << 8) | (average(b, n, inv) << 16) | 0xFF000000u;
+}
+
+// Views without dilation.
 __global__ void k_resolve(CloudView c, ViewTable vt, uint32_t view_base, Scratch s, bool publish) {
     const uint32_t v = blockIdx.y;
     if (v >= vt.n) return;
-    if (publish && v == 0 && blockIdx.x == 0) {
-        for (uint32_t i = threadIdx.x; i < vt.n * S_COUNT; i += blockDim.x) {
-            s.stats[(uint64_t)view_base * S_COUNT + i] = s.acc[i];
-            s.acc[i] = 0ull;
-        }
-        if (threadIdx.x < C_COUNT && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
-            s.counters[threadIdx.x] = 0u;
-    }
+    if (publish && v == 0 && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
     const ViewParams& vp = vt.v[v];
-    if (!vp.rgba) return;
+    if (!vp.rgba || (vp.flags & PC_VIEW_DILATE)) return;
     const uint64_t npix = (uint64_t)vp.width * vp.height;
-    const bool dilate = (vp.flags & PC_VIEW_DILATE) != 0;
     const uint32_t mode = vp.accum ? hqs_mode(vp.flags) : 0u;
     const unsigned long long empty = empty_key(vp.flags);
-    if (!dilate && !mode) {
+    if (!mode) {
         // plain resolve, 4 pixels per thread: two 16-byte key loads, four
         // independent colour gathers, one 16-byte store (vis and rgba are
         // 16-byte aligned); the last npix % 4 pixels one by one
@@ -1973,57 +2025,125 @@ __global__ void k_resolve(CloudView c, ViewTable vt, uint32_t view_base, Scratch
         return;
     }
     for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < npix;
-         p += (uint64_t)gridDim.x * blockDim.x) {
-        unsigned long long key = vp.vis[p];
-        uint64_t at = p;   // the pixel whose sums a shaded view shows
-        if (dilate) {
-            // Sec. 3.7: the closest point within (2r+1)^2 pixels, r by ring
-            const int px = (int)(p % vp.width), py = (int)(p / vp.width);
-            const int r = 1 + ring_of(__fadd_rn((float)px, 0.5f), __fadd_rn((float)py, 0.5f),
-                                      vp.width, vp.height);
-            const int x0 = max(px - r, 0), x1 = min(px + r, (int)vp.width - 1);
-            const int y0 = max(py - r, 0), y1 = min(py + r, (int)vp.height - 1);
-            for (int y = y0; y <= y1; ++y)
-                for (int x = x0; x <= x1; ++x) {
-                    const uint64_t q = (uint64_t)y * vp.width + x;
-                    const unsigned long long k = vp.vis[q];
-                    if (k < key) {
-                        key = k;
-                        at = q;
+         p += (uint64_t)gridDim.x * blockDim.x)
+        vp.rgba[p] = pixel_colour(c, vp, npix, mode, vp.vis[p], p, empty, s);
+}
+
+// Depth-aware dilation (Sec. 3.7): each pixel shows the closest point within
+// (2r+1)^2 pixels, r = 1, 2 or 3 by the pixel's ring. A block takes a tile of
+// kTile x kTile pixels: the keys with a border of 3 go to shared memory once, as
+// depths and indices, and the window's smallest depth is taken along the rows,
+// then along the columns, for each r that the tile has (one or two). The pixel it
+// belongs to is looked up in its row; equal depths, which the index settles, are
+// rare and cost a second look. Bound by instruction issue: 64-bit keys
+// compared the same way take twice the instructions. Two
+// 2016x2240 views: 213 us with every thread reading its own window (up to 49
+// keys through L1), 103 us with 64-bit keys in shared memory, 80 us this way.
+constexpr int kTile = 32, kBorder = 3, kTileIn = kTile + 2 * kBorder;
+
+struct DilateTile {
+    uint32_t depth[kTileIn][kTileIn], index[kTileIn][kTileIn];
+    uint32_t row[kTileIn][kTile];   // smallest depth of a row's window
+    uint32_t used;                  // bit r: some pixel of the tile has radius r
+};
+
+// The pixels of radius R of this thread's column (tx) and rows (ty + 8 j).
+template <int R>
+__device__ __forceinline__ void dilate_pixels(DilateTile& t, const uint32_t (&radius)[4], int tx, int ty,
+                                              int ox, int oy, const CloudView& c, const ViewParams& vp,
+                                              uint32_t mode, unsigned long long empty, const Scratch& s) {
+    for (int y = ty; y < kTileIn; y += 8) {
+        uint32_t m = t.depth[y][tx + kBorder - R];
+#pragma unroll
+        for (int d = -R + 1; d <= R; ++d) m = min(m, t.depth[y][tx + kBorder + d]);
+        t.row[y][tx] = m;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (radius[j] != R) continue;
+        const int y = ty + 8 * j + kBorder;
+        uint32_t row[2 * R + 1], m = ~0u;
+#pragma unroll
+        for (int d = 0; d <= 2 * R; ++d) m = min(m, row[d] = t.row[y + d - R][tx]);
+        uint32_t rows = 0;   // the window's rows with that depth, bit by bit
+#pragma unroll
+        for (int d = 0; d <= 2 * R; ++d) rows |= (uint32_t)(row[d] == m) << d;
+        // the pixel of that depth, of the smallest index where there are several
+        auto columns = [&](int yy) {
+            uint32_t cols = 0;
+#pragma unroll
+            for (int e = 0; e <= 2 * R; ++e)
+                cols |= (uint32_t)(t.depth[yy][tx + kBorder - R + e] == m) << e;
+            return cols;
+        };
+        int at_y = y - R + __ffs(rows) - 1;
+        uint32_t cols = columns(at_y);
+        int at_x = tx + kBorder - R + __ffs(cols) - 1;
+        uint32_t index = t.index[at_y][at_x];
+        if (((rows & (rows - 1u)) | (cols & (cols - 1u))) && m != (uint32_t)(empty >> 32)) {
+            for (; rows; rows &= rows - 1u) {
+                const int yy = y - R + __ffs(rows) - 1;
+                for (cols = columns(yy); cols; cols &= cols - 1u) {
+                    const int xx = tx + kBorder - R + __ffs(cols) - 1;
+                    if (t.index[yy][xx] < index) {
+                        index = t.index[yy][xx];
+                        at_x = xx;
+                        at_y = yy;
                     }
                 }
-        }
-        uint32_t out = 0u;
-        if (mode && key != empty) {
-            // Sec. 3.6: per-channel average of the sums, rounded down
-            uint32_t r, g, b, n;
-            const ulonglong2* two = reinterpret_cast<const ulonglong2*>(vp.accum);   // two-word sums
-            bool use_two = mode == 1;
-            if (mode == 2) {
-                use_two = (vp.accum[npix + (at >> 6)] >> (at & 63)) & 1ull;
-                two = reinterpret_cast<const ulonglong2*>(vp.accum + hqs_fallback_offset(npix));
-                const unsigned long long a = vp.accum[at];
-                r = (uint32_t)(a & 0x3FFFFu);
-                g = (uint32_t)((a >> 18) & 0x3FFFFu);
-                b = (uint32_t)((a >> 36) & 0x3FFFFu);
-                n = (uint32_t)(a >> 54);
             }
-            if (use_two) {
-                const ulonglong2 t = two[at];
-                r = (uint32_t)t.x;
-                g = (uint32_t)(t.x >> 32);
-                b = (uint32_t)t.y;
-                n = (uint32_t)(t.y >> 32);
-                if (n > kHqsMaxCount) raise_error(s, E_HQS_OVERFLOW, (uint32_t)at);
-            }
-            if (n) out = (r / n) | ((g / n) << 8) | ((b / n) << 16) | 0xFF000000u;
-        } else if (key != empty) {
-            const uint32_t idx = (uint32_t)key;
-            if (idx < c.n_points) out = c.color[idx];
-            else raise_error(s, E_INDEX_RANGE, idx);
         }
-        vp.rgba[p] = out;
+        const uint32_t W = vp.width;
+        const unsigned long long key = m == (uint32_t)(empty >> 32) ? empty
+                                       : ((unsigned long long)m << 32) | index;
+        const uint64_t at = (uint64_t)(oy + at_y - kBorder) * W + (uint32_t)(ox + at_x - kBorder);
+        vp.rgba[(uint64_t)(oy + ty + 8 * j) * W + (uint32_t)(ox + tx)] =
+            pixel_colour(c, vp, (uint64_t)W * vp.height, mode, key, at, empty, s);
     }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(256) k_resolve_dilated(CloudView c, ViewTable vt, uint32_t view_base,
+                                                       Scratch s, bool publish) {
+    if (publish && blockIdx.y == 0 && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
+    const ViewParams& vp = vt.v[blockIdx.y];
+    if (!vp.rgba || !(vp.flags & PC_VIEW_DILATE)) return;
+    const int W = (int)vp.width, H = (int)vp.height;
+    const int tiles_x = (W + kTile - 1) / kTile, tiles_y = (H + kTile - 1) / kTile;
+    if (blockIdx.x >= (uint32_t)(tiles_x * tiles_y)) return;
+    __shared__ DilateTile t;
+    const int ox = (int)(blockIdx.x % (uint32_t)tiles_x) * kTile;
+    const int oy = (int)(blockIdx.x / (uint32_t)tiles_x) * kTile;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int y = ty; y < kTileIn; y += 8)
+        for (int x = tx; x < kTileIn; x += 32) {
+            const int px = ox - kBorder + x, py = oy - kBorder + y;
+            const unsigned long long key =
+                px >= 0 && px < W && py >= 0 && py < H ? vp.vis[(uint64_t)py * W + px] : ~0ull;
+            t.depth[y][x] = (uint32_t)(key >> 32);
+            t.index[y][x] = (uint32_t)key;
+        }
+    uint32_t radius[4], any = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int x = ox + tx, y = oy + ty + 8 * j;
+        const bool inside = x < W && y < H;
+        radius[j] = inside ? 1u + (uint32_t)ring_of(__fadd_rn((float)x, 0.5f), __fadd_rn((float)y, 0.5f),
+                                                    vp.width, vp.height) : 0u;
+        if (inside) any |= 1u << radius[j];
+    }
+    if (threadIdx.x == 0) t.used = 0u;
+    __syncthreads();
+    any = __reduce_or_sync(FULL, any);
+    if (tx == 0) atomicOr(&t.used, any);
+    __syncthreads();
+    const uint32_t mode = vp.accum ? hqs_mode(vp.flags) : 0u;
+    const unsigned long long empty = empty_key(vp.flags);
+    const uint32_t used = t.used;
+    if (used & 2u) dilate_pixels<1>(t, radius, tx, ty, ox, oy, c, vp, mode, empty, s);
+    if (used & 4u) dilate_pixels<2>(t, radius, tx, ty, ox, oy, c, vp, mode, empty, s);
+    if (used & 8u) dilate_pixels<3>(t, radius, tx, ty, ox, oy, c, vp, mode, empty, s);
 }
 
 // ---- k_merge_min: element-wise minimum of two visibility buffers ------------------
@@ -2173,15 +2293,29 @@ cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cud
 }
 
 cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
-                           bool publish, cudaStream_t st) {
-    uint64_t maxpix = 0;
-    for (uint32_t v = 0; v < vt.n; ++v)
-        maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
+                           bool publish, cudaStream_t st, int* launched) {
+    uint64_t maxpix = 0, maxtiles = 0;
+    bool plain = false;
+    for (uint32_t v = 0; v < vt.n; ++v) {
+        const uint64_t w = vt.v[v].width, h = vt.v[v].height;
+        if (vt.v[v].flags & PC_VIEW_DILATE)
+            maxtiles = max(maxtiles, ((w + kTile - 1) / kTile) * ((h + kTile - 1) / kTile));
+        else
+            plain = true;
+        maxpix = max(maxpix, w * h);
+    }
+    *launched = (plain ? 1 : 0) + (maxtiles ? 1 : 0);
+    const unsigned views = vt.n ? vt.n : 1;
+    if (maxtiles) {   // at most 512 x 512 tiles
+        k_resolve_dilated<<<dim3((unsigned)maxtiles, views), 256, 0, st>>>(c, vt, view_base, s,
+                                                                        publish && !plain);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess || !plain) return e;
+    }
     const int threads = 256;
     uint64_t blocks = (maxpix + threads - 1) / threads;
     blocks = blocks < 1 ? 1 : (blocks > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : blocks);
-    dim3 grid((unsigned)blocks, vt.n ? vt.n : 1);
-    k_resolve<<<grid, threads, 0, st>>>(c, vt, view_base, s, publish);
+    k_resolve<<<dim3((unsigned)blocks, views), threads, 0, st>>>(c, vt, view_base, s, publish);
     return cudaGetLastError();
 }
 
