@@ -1333,6 +1333,17 @@ __device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counte
     return __shfl_sync(FULL, i, 0);
 }
 
+// The colour pass walks the list in another order: kFan places far apart in the
+// list in turn. Neighbouring entries add to the same pixels' sums, and the warps
+// that run at one time then wait for one another's reductions (200M-point
+// overview: 724 us in list order, 704 / 685 / 643 / 656 us with 8 / 64 / 1024 / 8192 places;
+// the depth pass gains nothing from it).
+constexpr uint32_t kFan = 1024u;
+__device__ __forceinline__ uint32_t fan_out(uint32_t i, uint32_t n) {
+    const uint32_t rounds = n / kFan;   // the places' lengths; the rest stays in order
+    return i < rounds * kFan ? (i % kFan) * rounds + i / kFan : i;
+}
+
 // Lengths of the draw list's two parts; none when they overflowed the buffer.
 __device__ __forceinline__ void entry_counts(const Scratch& s, uint32_t& front, uint32_t& back) {
     front = s.counters[C_ENTRIES];
@@ -1872,7 +1883,7 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, Scr
     n_entries += n_front;
     for (uint32_t i = first_entry(); i < n_entries;
          i = next_entry(s, FALLBACK ? C_GRAB_FALLBACK : C_GRAB_SHADE, n_entries, lane)) {
-        const DrawEntry e = s.entries[i < n_front ? i : s.capacity - 1u - (i - n_front)];
+        const DrawEntry e = s.entries[i < n_front ? fan_out(i, n_front) : s.capacity - 1u - (i - n_front)];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
