@@ -192,6 +192,18 @@ PCR_HD inline unsigned long long empty_key(uint32_t flags) {
 // resident at a block size.
 int raster_occupancy(int threads_per_block, uint32_t nviews);
 
+// ---- device encoder (encode.cu) ---------------------------------------------
+
+// Encodes n host points (0 < n < 2^32 - 1) into device buffers, with the bits of
+// encode_host; scratch: encode_device_scratch bytes of device memory. Returns when it is done;
+// *finite is false when some coordinate is NaN or infinite (the buffers then hold
+// nothing of use).
+uint64_t encode_device_scratch(uint64_t n, bool colours, bool keep_order);
+cudaError_t encode_device(const float* xyz, const uint32_t* rgba, uint64_t n, uint32_t batch_size,
+                          bool keep_order, void* scratch, pc_batch* batches, uint32_t* w1,
+                          uint32_t* w2, uint32_t* w3, uint32_t* color, cudaStream_t st,
+                          bool* finite);
+
 // ---- host encoder (encoder.cpp) -------------------------------------------
 
 pc_status encode_host(const float* xyz, const uint32_t* rgba, uint64_t n,
