@@ -124,10 +124,12 @@ pc_status pc_encode(const float* xyz, const uint32_t* rgba, uint64_t n,
                     uint32_t* w1, uint32_t* w2, uint32_t* w3, uint32_t* color,
                     uint32_t* perm);
 
-/* Encode host points (as pc_encode, batch size and PC_CFG_KEEP_ORDER from the
- * context's config) and
- * upload the cloud to device memory owned by the library. Synchronous. xyz and
- * rgba are read only during the call. *out receives a cloud handle. */
+/* Encode host points (with the bits of pc_encode; batch size and
+ * PC_CFG_KEEP_ORDER from the context's config) into a cloud in device memory owned
+ * by the library. The encoder runs on the device, with scratch memory of 40 bytes
+ * a point during the call, or on the host where the device has no room for
+ * it. Synchronous. xyz and rgba are read only during the call. *out receives a
+ * cloud handle. */
 pc_status pc_upload_cloud(pc_ctx* ctx, const float* xyz, const uint32_t* rgba,
                           uint64_t n, pc_cloud* out);
 
