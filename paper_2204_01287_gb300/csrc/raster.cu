@@ -1035,13 +1035,9 @@ __device__ __forceinline__ bool pixel_bracket(const FastView& fv, f2_t cxy, floa
 }
 
 // A lane's group of 4 decoded points of a certified batch in one view:
-// projection, pixel, early-depth reads and atomics. PARTIAL: only the points in
-// the mask valid are drawn (every word of the group decodes to a point that the
-// certificate covers, so the others only cost their arithmetic).
-template <bool PARTIAL>
+// projection, pixel, early-depth reads and atomics.
 __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_t (&xy)[4],
-                                                   const float (&z)[4], uint32_t g,
-                                                   uint32_t valid) {
+                                                   const float (&z)[4], uint32_t g) {
     f2_t cxy[4];
     float cw[4];
 #pragma unroll
@@ -1069,8 +1065,6 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
         pix[j] = min(by[j] * fv.width + bx[j] + fv.pixbias, fv.npix - 1u);
         w[j] = __float_as_uint(cw[j]);
         lim[j] = vis_hi[2ull * pix[j]];
-        // w is positive: a limit of 0 rejects the point
-        if (PARTIAL && !((valid >> j) & 1u)) lim[j] = 0u;
     }
     bool need = false;
 #pragma unroll
@@ -1088,6 +1082,145 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
     return n_atom;
 }
 
+// ---- one view: two points per packed instruction -------------------------------
+//
+// The one-view fast kernel packs two points instead of two rows: every operand is a
+// pair of points' values, so no half has to be copied to fill a pair, and the
+// view's coefficients come from the kernel's parameters as pairs (a, a). Every
+// operation and its order are those of the certified path above. 44.7 instead of 47.9
+// instructions a point; the raster pass of the 2B-point overview 3.30 -> 3.19 ms, of the
+// 200M-point one 383 -> 370 us.
+
+// The view's coefficients, each twice.
+struct PairView {
+    float2 x[4], y[4], w[4];   // clip rows: (m[r], m[r+4], m[r+8], m[r+12])
+    float2 W, H;
+    uint32_t width, npix, pixbias, pad;
+    unsigned long long* vis;
+};
+
+__device__ __forceinline__ f2_t f2_of(const float2& v) { return *reinterpret_cast<const f2_t*>(&v); }
+
+// Per-batch decode constants, each twice: c = min + fma(F, cell, nb).
+struct PairDec {
+    f2_t mn[3], cell[3], nb[3];
+};
+
+template <int K>
+__device__ __forceinline__ PairDec make_pair_dec(const pc_batch& b) {
+    PairDec d;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const float cell = ldexpf(b.size[a], -10 * K);
+        const float nb = -ldexpf(cell, K == 1 && a == 1 ? 13 : 23);
+        d.mn[a] = f2_pack(b.min[a], b.min[a]);
+        d.cell[a] = f2_pack(cell, cell);
+        d.nb[a] = f2_pack(nb, nb);
+    }
+    return d;
+}
+
+// The numbers F of a point's words (fast_decode).
+template <int K>
+__device__ __forceinline__ void fast_fields(uint32_t a, uint32_t b, uint32_t (&f)[3]) {
+    if (K == 1) {
+        f[0] = (a & 0x3FFu) | 0x4B000000u;
+        f[1] = (a & 0xFFC00u) | 0x46000000u;
+        f[2] = ((a >> 20) & 0x3FFu) | 0x4B000000u;
+    } else {
+        decode_q<2>(a, b, 0u, f[0], f[1], f[2]);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) f[i] |= 0x4B000000u;
+    }
+}
+
+__device__ __forceinline__ f2_t pair_row(const float2 (&m)[4], f2_t x, f2_t y, f2_t z) {
+    const f2_t zero = f2_pack(0.0f, 0.0f);
+    return f2_add(f2_add(f2_add(f2_fma_rn(f2_of(m[0]), x, zero), f2_fma_rn(f2_of(m[1]), y, zero)),
+                         f2_fma_rn(f2_of(m[2]), z, zero)),
+                  f2_of(m[3]));
+}
+
+// Two points (words a0, b0 and a1, b1): depths and pixel bits; false when a bracket
+// did not settle.
+template <int K>
+__device__ __forceinline__ bool pair_points(const PairView& v, const PairDec& d, uint32_t a0, uint32_t b0,
+                                            uint32_t a1, uint32_t b1, f2_t& cx, f2_t& cy, f2_t& cw,
+                                            f2_t& bx, f2_t& by) {
+    uint32_t f0[3], f1[3];
+    fast_fields<K>(a0, b0, f0);
+    fast_fields<K>(a1, b1, f1);
+    f2_t p[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        p[a] = f2_add(d.mn[a], f2_fma_rn(f2_pack(__uint_as_float(f0[a]), __uint_as_float(f1[a])), d.cell[a], d.nb[a]));
+    cx = pair_row(v.x, p[0], p[1], p[2]);
+    cy = pair_row(v.y, p[0], p[1], p[2]);
+    cw = pair_row(v.w, p[0], p[1], p[2]);
+    float w0, w1;
+    f2_unpack(cw, w0, w1);
+    const f2_t r = f2_pack(rcp_approx(w0), rcp_approx(w1));
+    const f2_t qx = f2_mul(cx, r), qy = f2_mul(cy, r);
+    const f2_t half = f2_pack(0.5f, 0.5f), magic = f2_pack(8388608.0f, 8388608.0f);
+    const f2_t below = f2_pack(0.5f - 0x1.0p-21f, 0.5f - 0x1.0p-21f);
+    const f2_t above = f2_pack(0.5f + 0x1.0p-21f, 0.5f + 0x1.0p-21f);
+    bx = f2_fma_rd(f2_fma_rn(qx, half, below), f2_of(v.W), magic);
+    by = f2_fma_rd(f2_fma_rn(qy, half, below), f2_of(v.H), magic);
+    return bx == f2_fma_rd(f2_fma_rn(qx, half, above), f2_of(v.W), magic) &&
+           by == f2_fma_rd(f2_fma_rn(qy, half, above), f2_of(v.H), magic);
+}
+
+// A lane's group of 4 points of a certified batch (as raster_decoded). PARTIAL: only
+// the points in the mask valid are drawn (every word of the group decodes to a
+// point that the certificate covers, so the others only cost their arithmetic).
+template <int K, bool PARTIAL>
+__device__ __forceinline__ uint32_t raster_pairs(const PairView& v, const PairDec& d, const uint4& q1,
+                                                 const uint4& q2, uint32_t g, uint32_t valid) {
+    f2_t cx[2], cy[2], cw[2], bx[2], by[2];
+    bool sure = pair_points<K>(v, d, q1.x, q2.x, q1.y, q2.y, cx[0], cy[0], cw[0], bx[0], by[0]);
+    sure &= pair_points<K>(v, d, q1.z, q2.z, q1.w, q2.w, cx[1], cy[1], cw[1], bx[1], by[1]);
+    uint32_t px[4], py[4], w[4], pix[4], lim[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int h = (j & 1) * 32;
+        px[j] = (uint32_t)(bx[j >> 1] >> h);
+        py[j] = (uint32_t)(by[j >> 1] >> h);
+        w[j] = (uint32_t)(cw[j >> 1] >> h);
+    }
+    if (!sure) {
+        // a bracket did not settle: the definition for all four (rare)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int h = (j & 1) * 32;
+            px[j] = exact_floor_bits(__uint_as_float((uint32_t)(cx[j >> 1] >> h)), __uint_as_float(w[j]), v.W.x);
+            py[j] = exact_floor_bits(__uint_as_float((uint32_t)(cy[j >> 1] >> h)), __uint_as_float(w[j]), v.H.x);
+        }
+    }
+    const uint32_t* vis_hi = reinterpret_cast<const uint32_t*>(v.vis) + 1;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        // inside the view by the certificate; the index is clamped all the same
+        pix[j] = min(py[j] * v.width + px[j] + v.pixbias, v.npix - 1u);
+        lim[j] = vis_hi[2ull * pix[j]];
+        // w is positive: a limit of 0 rejects the point
+        if (PARTIAL && !((valid >> j) & 1u)) lim[j] = 0u;
+    }
+    bool need = false;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) need |= w[j] <= lim[j];
+    if (!need) return 0;
+    uint32_t n_atom = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (w[j] <= lim[j]) {
+            atomicMin(v.vis + pix[j], ((unsigned long long)w[j] << 32) | (g + j));
+            ++n_atom;
+            if (j < 3 && pix[j + 1] == pix[j]) lim[j + 1] = min(lim[j + 1], w[j] - 1u);
+        }
+    }
+    return n_atom;
+}
+
 // Decode of a lane's group of 4 points from its words (k <= 2).
 template <int K>
 __device__ __forceinline__ void decode_group(const FastDec& d, const uint4& q1, const uint4& q2,
@@ -1098,24 +1231,13 @@ __device__ __forceinline__ void decode_group(const FastDec& d, const uint4& q1, 
     fast_decode<K>(d, q1.w, q2.w, xy[3], z[3]);
 }
 
-// One lane's group of 4 points of a certified batch, its words given.
-template <int K, bool PARTIAL>
-__device__ __forceinline__ uint32_t raster_group_fast(const FastView& fv, const FastDec& d,
-                                                      const uint4& q1, const uint4& q2,
-                                                      uint32_t g, uint32_t valid) {
-    f2_t xy[4];
-    float z[4];
-    decode_group<K>(d, q1, q2, xy, z);
-    return raster_decoded<PARTIAL>(fv, xy, z, g, valid);
-}
-
 // Points [p0, p1) of a certified batch at precision K (1 or 2). A lane loads the
 // words of its next step while it projects the current one, so the load's
 // latency hides behind that step's arithmetic. The depth reads are not moved
 // ahead: a read issued before the previous step's atomics would miss their
 // updates, and the extra atomics cost more than the latency saved.
 template <int K, bool STREAM>
-__device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const FastView& fv,
+__device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const PairView& fv,
                                                  const pc_batch& bt, uint32_t p0, uint32_t p1,
                                                  uint32_t lane) {
     uint32_t n_atom = 0;
@@ -1125,7 +1247,7 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const FastV
         prefetch_l2(c.w1 + base, bytes);
         if (K >= 2) prefetch_l2(c.w2 + base, bytes);
     }
-    const FastDec d = make_fast_dec<K>(bt);
+    const PairDec d = make_pair_dec<K>(bt);
     // the ragged first and last steps
     auto partial = [&](uint32_t g) {
         if (g >= p1) return;
@@ -1134,7 +1256,7 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const FastV
         for (int j = 0; j < 4; ++j) valid |= (uint32_t)(g + j >= p0 && g + j < p1) << j;
         const uint4 q1 = ld_words<STREAM>(c.w1 + g);
         const uint4 q2 = K >= 2 ? ld_words<STREAM>(c.w2 + g) : make_uint4(0, 0, 0, 0);
-        n_atom += raster_group_fast<K, true>(fv, d, q1, q2, g, valid);
+        n_atom += raster_pairs<K, true>(fv, d, q1, q2, g, valid);
     };
     if (base != p0 && base < p1) {
         partial(base + 4u * lane);
@@ -1160,10 +1282,10 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const FastV
                 a2 += 128;
                 n2 = ld_words<STREAM>(a2);
             }
-            n_atom += raster_group_fast<K, false>(fv, d, q1, q2, g, 0xFu);
+            n_atom += raster_pairs<K, false>(fv, d, q1, q2, g, 0xFu);
             g += 128u;
         }
-        n_atom += raster_group_fast<K, false>(fv, d, n1, n2, g, 0xFu);
+        n_atom += raster_pairs<K, false>(fv, d, n1, n2, g, 0xFu);
         base += nsteps << 7;
     }
     if (base < p1) partial(base + 4u * lane);
@@ -1222,7 +1344,7 @@ __device__ __forceinline__ void segment_fast_views(const CloudView& c, const Vie
             decode_group<K>(d, q1, q2, xy, z);
             for (uint32_t mm = vmask; mm; mm &= mm - 1) {
                 const uint32_t v = __ffs(mm) - 1;
-                const uint32_t n = raster_decoded<false>(make_fast_view(vt.v[v]), xy, z, g, 0xFu);
+                const uint32_t n = raster_decoded(make_fast_view(vt.v[v]), xy, z, g);
                 if (n) atomicAdd(&sh_atom[v], n);
             }
         }
@@ -1286,8 +1408,8 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
             f2_t xy[4];
             float z[4];
             decode_group<K>(d, q1, q2, xy, z);
-            if (vmask & 1u) na0 += raster_decoded<false>(make_fast_view(vt.v[0]), xy, z, g, 0xFu);
-            if (vmask & 2u) na1 += raster_decoded<false>(make_fast_view(vt.v[1]), xy, z, g, 0xFu);
+            if (vmask & 1u) na0 += raster_decoded(make_fast_view(vt.v[0]), xy, z, g);
+            if (vmask & 2u) na1 += raster_decoded(make_fast_view(vt.v[1]), xy, z, g);
         };
         for (uint32_t st = 1; st < nsteps; ++st) {
             const uint4 q1 = n1, q2 = n2;
@@ -1381,12 +1503,12 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
 
 // Five blocks of 256 threads per SM (48 registers): the depth reads' latency is
 // hidden by other warps, and more warps hide more of it.
-__global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c, ViewTable vt,
+__global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
+                                                               const __grid_constant__ PairView fv,
                                                                Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
-    const FastView fv = make_fast_view(vt.v[0]);
     uint32_t n_atom = 0;
     for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
         const DrawEntry e = s.entries[i];
@@ -2203,8 +2325,9 @@ cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cud
     uint64_t maxpix = 0;
     for (uint32_t v = 0; v < vt.n; ++v)
         maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
-    uint64_t parts = (maxpix / 2 + kCullThreads - 1) / kCullThreads;
-    parts = parts < 1 ? 1 : (parts > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : parts);
+    // the views share eight clearing blocks per SM
+    const uint64_t most = std::max<uint64_t>(1, (uint64_t)num_sms() * 8 / std::max(1u, vt.n));
+    const uint64_t parts = std::min(most, std::max<uint64_t>(1, (maxpix / 2 + kCullThreads - 1) / kCullThreads));
     const uint32_t per = cull_batches_per_block(c.n_batches, vt.n);
     const uint32_t cull = (c.n_batches + per - 1) / per;
     k_begin<<<cull + (uint32_t)parts * vt.n, kCullThreads, 0, st>>>(c, vt, s, cull, per, (uint32_t)parts);
@@ -2249,7 +2372,20 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
     cfg.stream = st;
     cfg.attrs = &early;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, vt, s);
+    const ViewParams& v = vt.v[0];
+    PairView pv{};
+    for (int j = 0; j < 4; ++j) {
+        pv.x[j] = make_float2(v.m[4 * j], v.m[4 * j]);
+        pv.y[j] = make_float2(v.m[4 * j + 1], v.m[4 * j + 1]);
+        pv.w[j] = make_float2(v.m[4 * j + 3], v.m[4 * j + 3]);
+    }
+    pv.W = make_float2((float)v.width, (float)v.width);
+    pv.H = make_float2((float)v.height, (float)v.height);
+    pv.width = v.width;
+    pv.npix = v.width * v.height;
+    pv.pixbias = 0u - 0x4B000000u * (v.width + 1u);
+    pv.vis = reinterpret_cast<unsigned long long*>(v.vis);
+    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, pv, s);
 }
 
 template <int LAYOUTS>
