@@ -23,7 +23,9 @@
 // m12; f = ((c / w) * 0.5 + 0.5) * W with an IEEE divide), or a packed f32x2
 // instruction that rounds each half the same way. The file is also compiled
 // with --fmad=false so nothing else is contracted.
+#include <algorithm>
 #include <cstdint>
+#include <utility>
 
 #include "pc_internal.h"
 
@@ -36,6 +38,14 @@ constexpr unsigned FULL = 0xFFFFFFFFu;
 __device__ __forceinline__ void raise_error(Scratch s, uint32_t code, uint32_t info) {
     if (atomicCAS(&s.counters[C_ERROR], 0u, code) == 0u) s.counters[C_ERRINFO] = info;
 }
+
+// A frame's kernels are launched so that each may start before the one before it
+// in the stream has ended (programmatic launch): its blocks are scheduled and its
+// code and parameters fetched while the other drains, and it waits here before
+// it touches memory. A frame of a 10M-point cloud 32.1 -> 25.3 us, an LOD frame
+// 38.4 -> 29.5 us, a 100M-point fly-through 86.2 -> 79.3 us.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- clear --------------------------------------------------------------------
 
@@ -451,6 +461,8 @@ __device__ __forceinline__ void init_cull(CullShared& sh, uint32_t nviews) {
 __global__ void __launch_bounds__(kCullThreads, 4) k_begin(CloudView c, ViewTable vt, Scratch s,
                                                       uint32_t cull_blocks, uint32_t per_block,
                                                       uint32_t clear_parts) {
+    start_next();
+    wait_for_previous();
     if (blockIdx.x >= cull_blocks) {
         const uint32_t j = blockIdx.x - cull_blocks;
         clear_view(vt.v[j / clear_parts], j % clear_parts, clear_parts);
@@ -497,8 +509,10 @@ __global__ void __launch_bounds__(kCullThreads, 4) k_begin(CloudView c, ViewTabl
 // (parents come first in breadth-first order; the root is its own parent).
 __global__ void __launch_bounds__(kCullThreads) k_lod_append(CloudView c, ViewTable vt, Scratch s,
                                                            uint32_t per_block) {
+    start_next();
     __shared__ CullShared sh;
     init_cull(sh, vt.n);
+    wait_for_previous();
     __syncthreads();
     const uint32_t first = blockIdx.x * per_block, n = min(per_block, c.n_batches - first);
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
@@ -1438,15 +1452,21 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
 
 constexpr int kRasterThreads = 256;
 
-// How the persistent warps share a list of n entries: a warp's first entry is
-// its own index in the grid, and only the entries past the grid's warps are
-// taken from a counter. A list that the grid covers in one round takes no
-// atomic; with one atomic per entry and one more per warp to see the end,
+// How the persistent warps share a list of n entries: each block's warps start
+// with neighbouring entries of its own, and only the entries past the grid's
+// warps are taken from a counter. A list that the grid covers in one round takes
+// no atomic; with one atomic per entry and one more per warp to see the end,
 // thousands of returning atomics on one address were the bound of small frames
-// (raster pass of an LOD frame of 1.3M points 26 us, 17 us this way).
+// (raster pass of an LOD frame of 1.3M points 26 us, 17 us this way). A short
+// list is spread over the blocks, but no thinner than four neighbours, which
+// share their pixels' lines in L1 (16 views of 1M points: a frame in 96 us when full
+// blocks take the list's 1,960 entries, 87 us with four each; the LOD frame
+// 29.7 us with full blocks, 30.4 us with four each, 33.6 us as thin as it goes).
 __device__ __forceinline__ uint32_t grid_warps() { return gridDim.x * (blockDim.x >> 5); }
-__device__ __forceinline__ uint32_t first_entry() {
-    return __shfl_sync(FULL, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), 0);
+__device__ __forceinline__ uint32_t first_entry(uint32_t n) {
+    const uint32_t per_block = blockDim.x >> 5, w = threadIdx.x >> 5;
+    const uint32_t share = min(per_block, max(4u, (n + gridDim.x - 1u) / gridDim.x));
+    return __shfl_sync(FULL, w < share ? blockIdx.x * share + w : n, 0);
 }
 __device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counter, uint32_t n,
                                                uint32_t lane) {
@@ -1506,11 +1526,12 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
 __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
                                                                const __grid_constant__ PairView fv,
                                                                Scratch s) {
+    start_next();
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
     uint32_t n_atom = 0;
-    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+    for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
         const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
@@ -1523,18 +1544,20 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
     }
     flush_atomics(s, 0u, n_atom, lane);
     // what follows in the stream waits for this kernel: it ends after the other
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    wait_for_previous();
 }
 
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView c, ViewTable vt,
                                                                   Scratch s) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // the fast kernel may start once the draw list is there
+    wait_for_previous();
+    start_next();
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_front, n_entries;
     entry_counts(s, n_front, n_entries);
     const ViewConst vc = make_view_const(vt.v[0]);
     uint32_t n_atom = 0;
-    for (uint32_t i = first_entry(); i < n_entries;
+    for (uint32_t i = first_entry(n_entries); i < n_entries;
          i = next_entry(s, C_GRAB_GENERAL, n_entries, lane)) {
         const DrawEntry e = s.entries[s.capacity - 1u - i];
         if (e.batch >= c.n_batches) {
@@ -1554,10 +1577,12 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView 
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, ViewTable vt,
                                                            Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
+    start_next();
+    wait_for_previous();
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
     uint32_t na0 = 0, na1 = 0;
-    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+    for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
         const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
@@ -1596,12 +1621,14 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, View
 __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, ViewTable vt,
                                                            Scratch s) {
     __shared__ uint32_t sh_atom[kMaxViewsPerLaunch];
+    start_next();
     for (uint32_t i = threadIdx.x; i < kMaxViewsPerLaunch; i += blockDim.x) sh_atom[i] = 0;
     __syncthreads();
+    wait_for_previous();
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
-    for (uint32_t i = first_entry(); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+    for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
         const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
@@ -2003,7 +2030,7 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, Scr
     uint32_t n_front, n_entries;
     entry_counts(s, n_front, n_entries);
     n_entries += n_front;
-    for (uint32_t i = first_entry(); i < n_entries;
+    for (uint32_t i = first_entry(n_entries); i < n_entries;
          i = next_entry(s, FALLBACK ? C_GRAB_FALLBACK : C_GRAB_SHADE, n_entries, lane)) {
         const DrawEntry e = s.entries[i < n_front ? fan_out(i, n_front) : s.capacity - 1u - (i - n_front)];
         if (e.batch >= c.n_batches) {
@@ -2113,6 +2140,8 @@ __device__ __forceinline__ uint32_t pixel_colour(const CloudView& c, const ViewP
 
 // Views without dilation.
 __global__ void k_resolve(CloudView c, ViewTable vt, uint32_t view_base, Scratch s, bool publish) {
+    start_next();
+    wait_for_previous();
     const uint32_t v = blockIdx.y;
     if (v >= vt.n) return;
     if (publish && v == 0 && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
@@ -2239,6 +2268,8 @@ __device__ __forceinline__ void dilate_pixels(DilateTile& t, const uint32_t (&ra
 
 __global__ void __launch_bounds__(256) k_resolve_dilated(CloudView c, ViewTable vt, uint32_t view_base,
                                                        Scratch s, bool publish) {
+    start_next();
+    wait_for_previous();
     if (publish && blockIdx.y == 0 && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
     const ViewParams& vp = vt.v[blockIdx.y];
     if (!vp.rgba || !(vp.flags & PC_VIEW_DILATE)) return;
@@ -2311,6 +2342,28 @@ int num_sms() {
 
 }  // namespace
 
+// Launch that may start early (wait_for_previous).
+template <class... Params, class... Args>
+static cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, unsigned threads, cudaStream_t st,
+                                Args&&... args) {
+    cudaLaunchAttribute early{};
+    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    // Blocks that wait hold their SM's slots. Captured launches get plain edges,
+    // since graphs are what programs replay on several streams at once (16 views of
+    // 1M points on three streams: 80 us a frame with early starts, 66 us without; one
+    // view of 10M points on one stream: 28 and 30 us).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &capture);
+    cfg.attrs = &early;
+    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // Batches per block of the cull pass: one round of its teams (fewer batches for
 // more views, so that a small cloud still spreads over the SMs), more when the
 // cloud has enough batches for four blocks per SM all the same (fewer blocks add
@@ -2330,15 +2383,14 @@ cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cud
     const uint64_t parts = std::min(most, std::max<uint64_t>(1, (maxpix / 2 + kCullThreads - 1) / kCullThreads));
     const uint32_t per = cull_batches_per_block(c.n_batches, vt.n);
     const uint32_t cull = (c.n_batches + per - 1) / per;
-    k_begin<<<cull + (uint32_t)parts * vt.n, kCullThreads, 0, st>>>(c, vt, s, cull, per, (uint32_t)parts);
-    return cudaGetLastError();
+    return launch_early(k_begin, dim3(cull + (uint32_t)parts * vt.n), kCullThreads, st, c, vt, s, cull, per,
+                        (uint32_t)parts);
 }
 
 cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
     if (c.n_batches == 0) return cudaSuccess;
     const uint32_t per = cull_batches_per_block(c.n_batches, 1);
-    k_lod_append<<<(c.n_batches + per - 1) / per, kCullThreads, 0, st>>>(c, vt, s, per);
-    return cudaGetLastError();
+    return launch_early(k_lod_append, dim3((c.n_batches + per - 1) / per), kCullThreads, st, c, vt, s, per);
 }
 
 int raster_occupancy(int threads_per_block, uint32_t nviews) {
@@ -2357,21 +2409,10 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
     threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
     const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
     *launched = vt.n == 1 ? 2 : 1;
-    if (vt.n > 2) k_rasterN<<<blocks, threads, 0, st>>>(c, vt, s);
-    else if (vt.n == 2) k_raster2<<<blocks, threads, 0, st>>>(c, vt, s);
-    if (vt.n != 1) return cudaGetLastError();
-    k_raster_general<<<num_sms() * 4, kRasterThreads, 0, st>>>(c, vt, s);
-    cudaError_t e = cudaGetLastError();
+    if (vt.n > 2) return launch_early(k_rasterN, dim3(blocks), threads, st, c, vt, s);
+    if (vt.n == 2) return launch_early(k_raster2, dim3(blocks), threads, st, c, vt, s);
+    cudaError_t e = launch_early(k_raster_general, dim3(num_sms() * 4), kRasterThreads, st, c, vt, s);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute early{};
-    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = st;
-    cfg.attrs = &early;
-    cfg.numAttrs = 1;
     const ViewParams& v = vt.v[0];
     PairView pv{};
     for (int j = 0; j < 4; ++j) {
@@ -2385,7 +2426,7 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
     pv.npix = v.width * v.height;
     pv.pixbias = 0u - 0x4B000000u * (v.width + 1u);
     pv.vis = reinterpret_cast<unsigned long long*>(v.vis);
-    return cudaLaunchKernelEx(&cfg, k_raster_fast, c, pv, s);
+    return launch_early(k_raster_fast, dim3(blocks), threads, st, c, pv, s);
 }
 
 template <int LAYOUTS>
@@ -2442,28 +2483,28 @@ cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cud
 cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
                            bool publish, cudaStream_t st, int* launched) {
     uint64_t maxpix = 0, maxtiles = 0;
-    bool plain = false;
+    bool plain = false, shaded = false;
     for (uint32_t v = 0; v < vt.n; ++v) {
         const uint64_t w = vt.v[v].width, h = vt.v[v].height;
         if (vt.v[v].flags & PC_VIEW_DILATE)
             maxtiles = max(maxtiles, ((w + kTile - 1) / kTile) * ((h + kTile - 1) / kTile));
         else
             plain = true;
+        shaded |= vt.v[v].accum != nullptr;
         maxpix = max(maxpix, w * h);
     }
     *launched = (plain ? 1 : 0) + (maxtiles ? 1 : 0);
     const unsigned views = vt.n ? vt.n : 1;
     if (maxtiles) {   // at most 512 x 512 tiles
-        k_resolve_dilated<<<dim3((unsigned)maxtiles, views), 256, 0, st>>>(c, vt, view_base, s,
-                                                                        publish && !plain);
-        const cudaError_t e = cudaGetLastError();
+        const cudaError_t e = launch_early(k_resolve_dilated, dim3((unsigned)maxtiles, views), 256, st, c, vt,
+                                           view_base, s, publish && !plain);
         if (e != cudaSuccess || !plain) return e;
     }
-    const int threads = 256;
-    uint64_t blocks = (maxpix + threads - 1) / threads;
-    blocks = blocks < 1 ? 1 : (blocks > (uint64_t)num_sms() * 8 ? (uint64_t)num_sms() * 8 : blocks);
-    k_resolve<<<dim3((unsigned)blocks, views), threads, 0, st>>>(c, vt, view_base, s, publish);
-    return cudaGetLastError();
+    // one or four pixels per thread
+    const uint64_t per_block = 256ull * (shaded ? 1 : 4);
+    const uint64_t blocks = std::min<uint64_t>((uint64_t)num_sms() * 8,
+                                               std::max<uint64_t>(1, (maxpix + per_block - 1) / per_block));
+    return launch_early(k_resolve, dim3((unsigned)blocks, views), 256, st, c, vt, view_base, s, publish);
 }
 
 }  // namespace pcr
