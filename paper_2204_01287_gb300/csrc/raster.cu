@@ -1628,8 +1628,18 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_rasterN(CloudView c, View
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_entries, n_back;
     entry_counts(s, n_entries, n_back);
+    // a list shorter than half the grid's warps: an entry's views go to 2^split
+    // warps, every 2^split-th view to each and four at least (16 views of 1M points,
+    // 1,960 entries for 4,864 warps: 76 -> 59 us). An entry's views otherwise stay with one
+    // warp, which then finds its words in cache and decodes them once: an entry
+    // per view took 104 us here, and 179 instead of 150 us for 8 views of 10M points.
+    uint32_t split = 0;
+    while ((n_entries << (split + 1)) <= grid_warps() && (vt.n >> (split + 1)) >= 4u) ++split;
+    n_entries <<= split;
+    const uint32_t part_views = split == 0u ? ~0u : split == 1u ? 0x55555555u : split == 2u ? 0x11111111u : 0x01010101u;
     for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
-        const DrawEntry e = s.entries[i];
+        DrawEntry e = s.entries[i >> split];
+        e.view_mask &= part_views << (i & ((1u << split) - 1u));
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
