@@ -841,6 +841,19 @@ __device__ __forceinline__ uint4 ld_words(const uint32_t* p) {
     return r;
 }
 
+// One lane's group of 4 points from its words: decode, raster.
+template <int K, bool PARTIAL>
+__device__ __forceinline__ uint32_t raster_words(const ViewConst& vc, const DecConst& d, const uint4& q1,
+                                                 const uint4& q2, const uint4& q3, uint32_t g,
+                                                 uint32_t valid) {
+    float x[4], y[4], z[4];
+    decode_point<K>(d, q1.x, q2.x, q3.x, x[0], y[0], z[0]);
+    decode_point<K>(d, q1.y, q2.y, q3.y, x[1], y[1], z[1]);
+    decode_point<K>(d, q1.z, q2.z, q3.z, x[2], y[2], z[2]);
+    decode_point<K>(d, q1.w, q2.w, q3.w, x[3], y[3], z[3]);
+    return raster_quad<PARTIAL>(vc, x, y, z, g, valid);
+}
+
 // Points [p0, p1) of one batch for one view at precision K. The loop over
 // groups of 4 is warp-uniform; STREAM loads bypass L1 (single view), the
 // multi-view kernel keeps the words in cache for the next view.
@@ -852,12 +865,7 @@ __device__ __forceinline__ uint32_t raster_group(const CloudView& c, const ViewC
     uint4 q2 = make_uint4(0, 0, 0, 0), q3 = make_uint4(0, 0, 0, 0);
     if (K >= 2) q2 = ld_words<STREAM>(c.w2 + g);
     if (K >= 3) q3 = ld_words<STREAM>(c.w3 + g);
-    float x[4], y[4], z[4];
-    decode_point<K>(d, q1.x, q2.x, q3.x, x[0], y[0], z[0]);
-    decode_point<K>(d, q1.y, q2.y, q3.y, x[1], y[1], z[1]);
-    decode_point<K>(d, q1.z, q2.z, q3.z, x[2], y[2], z[2]);
-    decode_point<K>(d, q1.w, q2.w, q3.w, x[3], y[3], z[3]);
-    return raster_quad<PARTIAL>(vc, x, y, z, g, valid);
+    return raster_words<K, PARTIAL>(vc, d, q1, q2, q3, g, valid);
 }
 
 // Points [p0, p1) of one batch for one view at precision K, 128 points per
@@ -894,8 +902,23 @@ __device__ __forceinline__ uint32_t segment(const CloudView& c, const ViewConst&
         }
         base += 128u;
     }
-    for (; base + 128u <= p1; base += 128u)
-        n_atom += raster_group<K, STREAM, false>(c, vc, d, base + 4u * lane, 0xFu);
+    if (base + 128u <= p1) {
+        // the next step's words are loaded while the current one is projected (a
+        // 100M-point fly-through frame 79.7 -> 76.9 us)
+        uint32_t g = base + 4u * lane;
+        uint4 n1 = ld_words<STREAM>(c.w1 + g), n2 = make_uint4(0, 0, 0, 0), n3 = n2;
+        if (K >= 2) n2 = ld_words<STREAM>(c.w2 + g);
+        if (K >= 3) n3 = ld_words<STREAM>(c.w3 + g);
+        for (; base + 128u <= p1; base += 128u, g += 128u) {
+            const uint4 q1 = n1, q2 = n2, q3 = n3;
+            if (base + 256u <= p1) {
+                n1 = ld_words<STREAM>(c.w1 + g + 128u);
+                if (K >= 2) n2 = ld_words<STREAM>(c.w2 + g + 128u);
+                if (K >= 3) n3 = ld_words<STREAM>(c.w3 + g + 128u);
+            }
+            n_atom += raster_words<K, false>(vc, d, q1, q2, q3, g, 0xFu);
+        }
+    }
     if (base < p1) {
         const uint32_t g = base + 4u * lane;
         if (g < p1) {
