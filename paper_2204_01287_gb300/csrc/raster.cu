@@ -1178,61 +1178,79 @@ __device__ __forceinline__ f2_t pair_row(const float2 (&m)[4], f2_t x, f2_t y, f
                   f2_of(m[3]));
 }
 
-// Two points (words a0, b0 and a1, b1): depths and pixel bits; false when a bracket
-// did not settle.
+// Decoded positions of a lane's group of 4 points, as two pairs per axis.
+struct PairPos {
+    f2_t x[2], y[2], z[2];
+};
+
 template <int K>
-__device__ __forceinline__ bool pair_points(const PairView& v, const PairDec& d, uint32_t a0, uint32_t b0,
-                                            uint32_t a1, uint32_t b1, f2_t& cx, f2_t& cy, f2_t& cw,
-                                            f2_t& bx, f2_t& by) {
-    uint32_t f0[3], f1[3];
-    fast_fields<K>(a0, b0, f0);
-    fast_fields<K>(a1, b1, f1);
-    f2_t p[3];
+__device__ __forceinline__ PairPos decode_pairs(const PairDec& d, const uint4& q1, const uint4& q2) {
+    const uint32_t a[4] = {q1.x, q1.y, q1.z, q1.w}, b[4] = {q2.x, q2.y, q2.z, q2.w};
+    PairPos p;
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
-        p[a] = f2_add(d.mn[a], f2_fma_rn(f2_pack(__uint_as_float(f0[a]), __uint_as_float(f1[a])), d.cell[a], d.nb[a]));
-    cx = pair_row(v.x, p[0], p[1], p[2]);
-    cy = pair_row(v.y, p[0], p[1], p[2]);
-    cw = pair_row(v.w, p[0], p[1], p[2]);
-    float w0, w1;
-    f2_unpack(cw, w0, w1);
-    const f2_t r = f2_pack(rcp_approx(w0), rcp_approx(w1));
-    const f2_t qx = f2_mul(cx, r), qy = f2_mul(cy, r);
+    for (int h = 0; h < 2; ++h) {
+        uint32_t f0[3], f1[3];
+        fast_fields<K>(a[2 * h], b[2 * h], f0);
+        fast_fields<K>(a[2 * h + 1], b[2 * h + 1], f1);
+        f2_t c[3];
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+            c[i] = f2_add(d.mn[i], f2_fma_rn(f2_pack(__uint_as_float(f0[i]), __uint_as_float(f1[i])),
+                                             d.cell[i], d.nb[i]));
+        p.x[h] = c[0];
+        p.y[h] = c[1];
+        p.z[h] = c[2];
+    }
+    return p;
+}
+
+// Depths (as bits) and floor bits of the pixels of a lane's group of 4 decoded points.
+__device__ __forceinline__ void project_pairs(const PairView& v, const PairPos& p, uint32_t (&w)[4],
+                                              uint32_t (&px)[4], uint32_t (&py)[4]) {
     const f2_t half = f2_pack(0.5f, 0.5f), magic = f2_pack(8388608.0f, 8388608.0f);
     const f2_t below = f2_pack(0.5f - 0x1.0p-21f, 0.5f - 0x1.0p-21f);
     const f2_t above = f2_pack(0.5f + 0x1.0p-21f, 0.5f + 0x1.0p-21f);
-    bx = f2_fma_rd(f2_fma_rn(qx, half, below), f2_of(v.W), magic);
-    by = f2_fma_rd(f2_fma_rn(qy, half, below), f2_of(v.H), magic);
-    return bx == f2_fma_rd(f2_fma_rn(qx, half, above), f2_of(v.W), magic) &&
-           by == f2_fma_rd(f2_fma_rn(qy, half, above), f2_of(v.H), magic);
-}
-
-// A lane's group of 4 points of a certified batch (as raster_decoded). PARTIAL: only
-// the points in the mask valid are drawn (every word of the group decodes to a
-// point that the certificate covers, so the others only cost their arithmetic).
-template <int K, bool PARTIAL>
-__device__ __forceinline__ uint32_t raster_pairs(const PairView& v, const PairDec& d, const uint4& q1,
-                                                 const uint4& q2, uint32_t g, uint32_t valid) {
-    f2_t cx[2], cy[2], cw[2], bx[2], by[2];
-    bool sure = pair_points<K>(v, d, q1.x, q2.x, q1.y, q2.y, cx[0], cy[0], cw[0], bx[0], by[0]);
-    sure &= pair_points<K>(v, d, q1.z, q2.z, q1.w, q2.w, cx[1], cy[1], cw[1], bx[1], by[1]);
-    uint32_t px[4], py[4], w[4], pix[4], lim[4];
+    f2_t cx[2], cy[2];
+    bool sure = true;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const int h = (j & 1) * 32;
-        px[j] = (uint32_t)(bx[j >> 1] >> h);
-        py[j] = (uint32_t)(by[j >> 1] >> h);
-        w[j] = (uint32_t)(cw[j >> 1] >> h);
+    for (int h = 0; h < 2; ++h) {
+        cx[h] = pair_row(v.x, p.x[h], p.y[h], p.z[h]);
+        cy[h] = pair_row(v.y, p.x[h], p.y[h], p.z[h]);
+        const f2_t cw = pair_row(v.w, p.x[h], p.y[h], p.z[h]);
+        float w0, w1;
+        f2_unpack(cw, w0, w1);
+        const f2_t r = f2_pack(rcp_approx(w0), rcp_approx(w1));
+        const f2_t qx = f2_mul(cx[h], r), qy = f2_mul(cy[h], r);
+        const f2_t bx = f2_fma_rd(f2_fma_rn(qx, half, below), f2_of(v.W), magic);
+        const f2_t by = f2_fma_rd(f2_fma_rn(qy, half, below), f2_of(v.H), magic);
+        sure = sure && bx == f2_fma_rd(f2_fma_rn(qx, half, above), f2_of(v.W), magic) &&
+               by == f2_fma_rd(f2_fma_rn(qy, half, above), f2_of(v.H), magic);
+        w[2 * h] = __float_as_uint(w0);
+        w[2 * h + 1] = __float_as_uint(w1);
+        px[2 * h] = (uint32_t)bx;
+        px[2 * h + 1] = (uint32_t)(bx >> 32);
+        py[2 * h] = (uint32_t)by;
+        py[2 * h + 1] = (uint32_t)(by >> 32);
     }
     if (!sure) {
         // a bracket did not settle: the definition for all four (rare)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int h = (j & 1) * 32;
-            px[j] = exact_floor_bits(__uint_as_float((uint32_t)(cx[j >> 1] >> h)), __uint_as_float(w[j]), v.W.x);
-            py[j] = exact_floor_bits(__uint_as_float((uint32_t)(cy[j >> 1] >> h)), __uint_as_float(w[j]), v.H.x);
+            const int s = (j & 1) * 32;
+            px[j] = exact_floor_bits(__uint_as_float((uint32_t)(cx[j >> 1] >> s)), __uint_as_float(w[j]), v.W.x);
+            py[j] = exact_floor_bits(__uint_as_float((uint32_t)(cy[j >> 1] >> s)), __uint_as_float(w[j]), v.H.x);
         }
     }
+}
+
+// A lane's group of 4 points of a certified batch (as raster_decoded). PARTIAL: only
+// the points in the mask valid are drawn (every word of the group decodes to a
+// point that the certificate covers, so the others only cost their arithmetic).
+template <bool PARTIAL>
+__device__ __forceinline__ uint32_t raster_pairs(const PairView& v, const PairPos& p, uint32_t g,
+                                                 uint32_t valid) {
+    uint32_t px[4], py[4], w[4], pix[4], lim[4];
+    project_pairs(v, p, w, px, py);
     const uint32_t* vis_hi = reinterpret_cast<const uint32_t*>(v.vis) + 1;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -1293,7 +1311,7 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const PairV
         for (int j = 0; j < 4; ++j) valid |= (uint32_t)(g + j >= p0 && g + j < p1) << j;
         const uint4 q1 = ld_words<STREAM>(c.w1 + g);
         const uint4 q2 = K >= 2 ? ld_words<STREAM>(c.w2 + g) : make_uint4(0, 0, 0, 0);
-        n_atom += raster_pairs<K, true>(fv, d, q1, q2, g, valid);
+        n_atom += raster_pairs<true>(fv, decode_pairs<K>(d, q1, q2), g, valid);
     };
     if (base != p0 && base < p1) {
         partial(base + 4u * lane);
@@ -1319,10 +1337,10 @@ __device__ __forceinline__ uint32_t segment_fast(const CloudView& c, const PairV
                 a2 += 128;
                 n2 = ld_words<STREAM>(a2);
             }
-            n_atom += raster_pairs<K, false>(fv, d, q1, q2, g, 0xFu);
+            n_atom += raster_pairs<false>(fv, decode_pairs<K>(d, q1, q2), g, 0xFu);
             g += 128u;
         }
-        n_atom += raster_pairs<K, false>(fv, d, n1, n2, g, 0xFu);
+        n_atom += raster_pairs<false>(fv, decode_pairs<K>(d, n1, n2), g, 0xFu);
         base += nsteps << 7;
     }
     if (base < p1) partial(base + 4u * lane);
@@ -1404,6 +1422,7 @@ __device__ __forceinline__ void segment_fast_views(const CloudView& c, const Vie
 // only known at run time makes them loads).
 template <int K>
 __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const ViewTable& vt,
+                                                  const PairView& v0, const PairView& v1,
                                                   uint32_t vmask, const pc_batch& bt,
                                                   uint32_t p0, uint32_t p1, uint32_t lane,
                                                   uint32_t& na0, uint32_t& na1) {
@@ -1433,7 +1452,7 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
         base += 128u;
     }
     if (base + 128u <= p1) {
-        const FastDec d = make_fast_dec<K>(bt);
+        const PairDec d = make_pair_dec<K>(bt);
         const uint32_t nsteps = (p1 - base) >> 7;
         uint32_t g = base + 4u * lane;
         const uint32_t* a1 = c.w1 + g;
@@ -1442,11 +1461,9 @@ __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const View
         uint4 n2 = make_uint4(0, 0, 0, 0);
         if (K >= 2) n2 = ld_words<true>(a2);
         auto step = [&](const uint4& q1, const uint4& q2) {
-            f2_t xy[4];
-            float z[4];
-            decode_group<K>(d, q1, q2, xy, z);
-            if (vmask & 1u) na0 += raster_decoded(make_fast_view(vt.v[0]), xy, z, g);
-            if (vmask & 2u) na1 += raster_decoded(make_fast_view(vt.v[1]), xy, z, g);
+            const PairPos p = decode_pairs<K>(d, q1, q2);
+            if (vmask & 1u) na0 += raster_pairs<false>(v0, p, g, 0xFu);
+            if (vmask & 2u) na1 += raster_pairs<false>(v1, p, g, 0xFu);
         };
         for (uint32_t st = 1; st < nsteps; ++st) {
             const uint4 q1 = n1, q2 = n2;
@@ -1598,6 +1615,8 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView 
 // views' constants at fixed parameter offsets. Four blocks of 256 threads per
 // SM (64 registers).
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, ViewTable vt,
+                                                           const __grid_constant__ PairView v0,
+                                                           const __grid_constant__ PairView v1,
                                                            Scratch s) {
     const uint32_t lane = threadIdx.x & 31;
     start_next();
@@ -1622,8 +1641,8 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster2(CloudView c, View
             if (k == 1) fast1 |= 1u << v;
             if (k == 2) fast2 |= 1u << v;
         }
-        if (fast1) segment_fast_pair<1>(c, vt, fast1, bt, p0, p1, lane, na0, na1);
-        if (fast2) segment_fast_pair<2>(c, vt, fast2, bt, p0, p1, lane, na0, na1);
+        if (fast1) segment_fast_pair<1>(c, vt, v0, v1, fast1, bt, p0, p1, lane, na0, na1);
+        if (fast2) segment_fast_pair<2>(c, vt, v0, v1, fast2, bt, p0, p1, lane, na0, na1);
         const uint32_t rest = e.view_mask & ~(fast1 | fast2);
         if (rest & 1u)
             na0 += segment_k<false>(c, make_view_const(vt.v[0]), bt, (int)(e.kcodes & 3u), p0, p1,
@@ -2436,17 +2455,7 @@ int raster_occupancy(int threads_per_block, uint32_t nviews) {
     return nb > 0 ? nb : 1;
 }
 
-cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
-                          RasterShape shape, cudaStream_t st, int* launched) {
-    int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
-    threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
-    const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
-    *launched = vt.n == 1 ? 2 : 1;
-    if (vt.n > 2) return launch_early(k_rasterN, dim3(blocks), threads, st, c, vt, s);
-    if (vt.n == 2) return launch_early(k_raster2, dim3(blocks), threads, st, c, vt, s);
-    cudaError_t e = launch_early(k_raster_general, dim3(num_sms() * 4), kRasterThreads, st, c, vt, s);
-    if (e != cudaSuccess) return e;
-    const ViewParams& v = vt.v[0];
+static PairView make_pair_view(const ViewParams& v) {
     PairView pv{};
     for (int j = 0; j < 4; ++j) {
         pv.x[j] = make_float2(v.m[4 * j], v.m[4 * j]);
@@ -2459,7 +2468,21 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
     pv.npix = v.width * v.height;
     pv.pixbias = 0u - 0x4B000000u * (v.width + 1u);
     pv.vis = reinterpret_cast<unsigned long long*>(v.vis);
-    return launch_early(k_raster_fast, dim3(blocks), threads, st, c, pv, s);
+    return pv;
+}
+
+cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
+                          RasterShape shape, cudaStream_t st, int* launched) {
+    int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
+    threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
+    const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
+    *launched = vt.n == 1 ? 2 : 1;
+    if (vt.n > 2) return launch_early(k_rasterN, dim3(blocks), threads, st, c, vt, s);
+    if (vt.n == 2) return launch_early(k_raster2, dim3(blocks), threads, st, c, vt, make_pair_view(vt.v[0]),
+                                         make_pair_view(vt.v[1]), s);
+    cudaError_t e = launch_early(k_raster_general, dim3(num_sms() * 4), kRasterThreads, st, c, vt, s);
+    if (e != cudaSuccess) return e;
+    return launch_early(k_raster_fast, dim3(blocks), threads, st, c, make_pair_view(vt.v[0]), s);
 }
 
 template <int LAYOUTS>
