@@ -68,7 +68,7 @@ __device__ __forceinline__ void clear_view(const ViewParams& vp, uint32_t part, 
     }
 }
 
-// ---- k_cull: Sec. 3.2 culling and Sec. 3.3 precision ----------------------------
+// ---- culling (Sec. 3.2) and precision (Sec. 3.3) --------------------------------
 
 // Row r of the clip transform at a position: ((m[r] x + m[r+4] y) + m[r+8] z) + m[r+12].
 __device__ __forceinline__ float clip_row(const float* m, int r, float x, float y, float z) {
@@ -255,8 +255,9 @@ __device__ __forceinline__ BatchTest test_batch(const pc_batch& b, const ViewPar
 #pragma unroll
     for (int a = 0; a < 4; ++a) R[a] = l <= 2u ? m[4 * a] : m[4 * a + 1];
     const float bw = row_mag32(Wr, lo, hi), br = row_mag32(R, lo, hi);
-    r.culled = false;
-    if (need_cull) {
+    // the ballots are for the whole warp, whose teams may have views with and
+    // without culling
+    {
         const float g = 6.0f * 0x1.0p-24f, band = 0x1.0p-16f;
         const float mag = l == 0u ? bw : __fadd_rn(br, __fmul_rn(e1, bw));
         float sp[4];
@@ -272,8 +273,8 @@ __device__ __forceinline__ BatchTest test_batch(const pc_batch& b, const ViewPar
         const bool out = __ballot_sync(FULL, test && t < -lim) & team;
         const bool open = __ballot_sync(FULL, test && !(t < -lim) && !(t > lim)) & team;
         // a plane decided as culling settles it; otherwise every plane must be decided
-        if (bad || (open && !out)) r.culled = cull_batch_exact(b, v);
-        else r.culled = out;
+        if (need_cull && (bad || (open && !out))) r.culled = cull_batch_exact(b, v);
+        else r.culled = need_cull && out;
     }
     // certificate
     {
@@ -393,6 +394,8 @@ __device__ void append_batches(CullShared& sh, uint32_t first, uint32_t n, const
         const uint64_t end = (base >> 32) + (uint32_t)base + (total >> 32) + (uint32_t)total;
         if (end > s.capacity) {
             if (nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)end);
+            // the counts must not come round to a sum that looks as if it fitted
+            if (lane == 31) atomicOr(&s.counters[C_GENERAL], 0x80000000u);
             nseg = 0;
         }
         if (i < n) {
@@ -931,7 +934,7 @@ __device__ __forceinline__ uint32_t segment(const CloudView& c, const ViewConst&
     return n_atom;
 }
 
-// ---- k_raster fast path: batches certified by batch_fast ----------------------
+// ---- k_raster fast path: certified batches (test_batch) -----------------------
 //
 // For a certified batch every point is in front of the eye with w in
 // [2^-99, 2^99] and its floor pixel lies inside the view, so the per-point
@@ -1417,7 +1420,7 @@ __device__ __forceinline__ void segment_fast_views(const CloudView& c, const Vie
 
 // Points [p0, p1) of a certified batch at precision K for views 0 and 1 of a
 // two-view launch (vmask: bit v set when view v is certified at K): one decode
-// per step as in segment_fast_views, then each view with its constants read at
+// per step as in segment_fast_views, two points per instruction, then each view with its constants read at
 // fixed parameter offsets, as in the one-view kernel (a view index that is
 // only known at run time makes them loads).
 template <int K>
@@ -1840,7 +1843,7 @@ __device__ __forceinline__ void shade_flush(ShadeRun& run, const ShadeBuf& sb, P
 // per step with 32-byte loads, each of which fills one sector (the cloud's
 // arrays are 32-byte aligned and padded past the last 8-point step); otherwise
 // 4 points per step with 16-byte loads.
-// FAST: a certified batch (batch_fast) at k <= 2, projected as in the depth
+// FAST: a certified batch (test_batch) at k <= 2, projected as in the depth
 // pass's fast path; every point is then in front of the eye and inside the view.
 template <int K, ShadeMode MODE, bool FAST>
 __device__ __forceinline__ uint32_t shade_segment(const CloudView& c, const ViewConst& vc,
@@ -2410,7 +2413,10 @@ static cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, unsigned t
     // 1M points on three streams: 80 us a frame with early starts, 66 us without; one
     // view of 10M points on one stream: 28 and 30 us).
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(st, &capture);
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
+        cudaGetLastError();   // plain edges are always right; the launch reports what is wrong
+        capture = cudaStreamCaptureStatusActive;
+    }
     cfg.attrs = &early;
     cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);

@@ -1,5 +1,5 @@
 /* Adversarial check of the fast-path certificate that the cull pass computes
- * for each batch and view (batch_fast in the raster kernels).
+ * for each batch and view (test_batch in the raster kernels).
  *
  * A certified batch skips the per-point tests of the general path, so the
  * certificate must be sound: every point the batch can decode to must be in

@@ -90,3 +90,28 @@ def test_statistics_survive_a_separate_resolve(cuda_lib):
         ctx.render(cloud, [v], fbs)
         torch.cuda.synchronize()
         assert ctx.stats()["points_k"] == st["points_k"]
+
+
+@pytest.mark.parametrize("nviews", [2, 3, 5, 8, 17])
+@pytest.mark.parametrize("n,batch", [(300, 8), (300_000, 10240)])
+def test_views_with_and_without_culling_share_a_warp(cuda_lib, n, batch, nviews):
+    """Views of one launch that differ in culling and forced precision: the
+    teams of a warp test batches for views of both kinds."""
+    import torch
+    p = S.terrain_params(4000.0, 0.2, 60)
+    xyz, rgba = S.terrain(n, p, seed=1)
+    enc = O.encode(xyz, rgba, batch)
+    W, H = 160, 90
+    with pcr.Context(0, batch_size=batch) as ctx:
+        cloud = ctx.upload(xyz, rgba)
+        ms = [S.flythrough(p, 10 * i, 120, W, H, seed=1) if i % 3 else S.cube_camera(W, H)
+              for i in range(nviews)]
+        ks = [i % 4 for i in range(nviews)]
+        views = [pcr.make_view(m, W, H, (pcr.PC_VIEW_CULL if i % 2 else 0) | pcr.PC_VIEW_FORCE_K(k))
+                 for i, (m, k) in enumerate(zip(ms, ks))]
+        fbs = ctx.render(cloud, views)
+        torch.cuda.synchronize()
+        for i, (m, k) in enumerate(zip(ms, ks)):
+            ovis, st = O.render(enc, O.make_view(m, W, H, cull=bool(i % 2), force_k=k))
+            assert np.array_equal(pcr.vis_to_numpy(fbs[i][0]), ovis), i
+            assert ctx.stats(i)["batches_k"] == st["batches_k"]
