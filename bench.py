@@ -39,12 +39,12 @@ sys.path.insert(0, ROOT)
 
 METRIC = "Gpoints/s & ms/frame at 2B pts 1080p; %HBM peak; batched views/s, p50/p99"
 
-# DRAM bytes (read + write) of one k_raster1 launch in the ncu capture of the
+# DRAM bytes (read + write) of the one-view raster kernels in the ncu capture of the
 # 50M-point overview (the summary under profiles/); the traffic of the bench's
 # launch is this scaled by the points processed. Re-capture when the kernel changes.
 NOMINAL_HBM_GBS = 7900.0   # GB300 HBM3e, nominal
 RASTER_CAPTURE_POINTS = 50_000_000
-RASTER_CAPTURE_DRAM_BYTES = 210_849_024
+RASTER_CAPTURE_DRAM_BYTES = 207_170_816
 
 
 def parse():

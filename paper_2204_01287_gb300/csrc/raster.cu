@@ -1127,8 +1127,8 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
 // The one-view fast kernel packs two points instead of two rows: every operand is a
 // pair of points' values, so no half has to be copied to fill a pair, and the
 // view's coefficients come from the kernel's parameters as pairs (a, a). Every
-// operation and its order are those of the certified path above. 44.7 instead of 47.9
-// instructions a point; the raster pass of the 2B-point overview 3.30 -> 3.19 ms, of the
+// operation and its order are those of the certified path above. On a view as dense
+// as the 2B-point frame 44.7 warp instructions per 32 points, about 47.5 before; the raster pass of the 2B-point overview 3.30 -> 3.19 ms, of the
 // 200M-point one 383 -> 370 us.
 
 // The view's coefficients, each twice.
