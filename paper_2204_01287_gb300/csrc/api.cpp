@@ -98,7 +98,7 @@ pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
             e = cudaMemsetAsync(s.scratch.counters, 0, sizeof(uint32_t) * C_ERROR, s.stream);
         if (e == cudaSuccess)
             e = cudaMemsetAsync(s.scratch.counters + C_ERRINFO + 1, 0,
-                                sizeof(uint32_t) * (C_COUNT - C_ERRINFO - 1), s.stream);
+                                sizeof(uint32_t) * (C_LIST - C_ERRINFO - 1), s.stream);
         if (e != cudaSuccess) return cuda_fail(e, "scratch reset");
         s.unclean = false;
     }
@@ -280,6 +280,7 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         }
         if (fe) cudaEventRecord(fe->ev[2], st);
         int raster_kernels = 0;
+        slot->scratch.frame = next_frame(slot->scratch.frame);
         e = launch_raster(cv, vt, slot->scratch, shape, st, &raster_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "raster launch");
         if (fe) cudaEventRecord(fe->ev[3], st);

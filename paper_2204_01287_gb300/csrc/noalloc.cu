@@ -6,6 +6,7 @@
 // from per-stream buffers that the library allocates; this entry point takes
 // it from a file-scope __device__ array instead, so that callers which may not
 // allocate device memory can still render.
+#include <atomic>
 #include <cstddef>
 #include <cstring>
 #include <mutex>
@@ -103,6 +104,8 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     s.acc = L->acc;
     s.stats = L->stats;
     s.lod_sel = nullptr;
+    static std::atomic<uint64_t> calls{0};   // numbers 1, 2, ... of the process's calls
+    s.frame = (uint32_t)(calls.fetch_add(1u) % 0xFFFFFFFFu) + 1u;
     // the array keeps the previous call's contents: counters and sums
     // (including the error flag) start from zero every call
     if (cudaMemsetAsync(L->counters, 0, sizeof L->counters + sizeof L->acc, st) != cudaSuccess)

@@ -29,7 +29,9 @@ enum : uint32_t {
     C_GRAB_FALLBACK = 5,  // ... by the second pass of packed shading
     C_GRAB = 6,      // entries taken by raster warps, past each warp's first
     C_GRAB_GENERAL = 7,   // ... by the general one-view kernel
-    C_COUNT = 8       // even: the scratch sums follow the counters
+    C_LIST = 8,       // 64 bits: frame number and C_ENTRIES, from the general one-view
+                      // kernel to the fast one
+    C_COUNT = 10      // even: the scratch sums follow the counters
 };
 
 // Per-view statistics slots in Scratch::stats (uint64 each).
@@ -151,10 +153,15 @@ struct Scratch {
     uint32_t* counters;   // C_COUNT
     unsigned long long* stats;  // kMaxViewsPerRender * S_COUNT: the last frame's
     unsigned long long* acc;    // kMaxViewsPerLaunch * S_COUNT: sums of the launch in
-                                // progress. acc and counters (the error words apart)
-                                // are zero between launches; k_resolve leaves them so
+                                // progress. acc and the counters before C_LIST (the
+                                // error words apart) are zero between launches;
+                                // k_resolve leaves them so
+    uint32_t frame;       // number of this launch (next_frame)
     LodSel* lod_sel;      // LOD: per node
 };
+
+// The number of the launch after `last`: any but 0, which a cleared scratch holds.
+inline uint32_t next_frame(uint32_t last) { return last == ~0u ? 1u : last + 1u; }
 
 // Launch-shape knobs for the raster kernel.
 struct RasterShape {

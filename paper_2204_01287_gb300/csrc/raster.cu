@@ -42,7 +42,8 @@ __device__ __forceinline__ void raise_error(Scratch s, uint32_t code, uint32_t i
 // A frame's kernels are launched so that each may start before the one before it
 // in the stream has ended (programmatic launch): its blocks are scheduled and its
 // code and parameters fetched while the other drains, and it waits here before
-// it touches memory. A frame of a 10M-point cloud 32.1 -> 25.3 us, an LOD frame
+// it touches memory that a kernel of the stream writes. One kernel, k_raster_fast,
+// may go on without waiting (take_list). A frame of a 10M-point cloud 32.1 -> 25.3 us, an LOD frame
 // 38.4 -> 29.5 us, a 100M-point fly-through 86.2 -> 79.3 us.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -1536,6 +1537,37 @@ __device__ __forceinline__ void entry_counts(const Scratch& s, uint32_t& front, 
     if ((uint64_t)front + back > s.capacity) front = back = 0;
 }
 
+// The draw list's way from k_raster_general to k_raster_fast, which runs beside it
+// and so cannot wait for it to end. k_raster_general has waited for the first pass;
+// one thread of it then stores the frame's number with the front's length
+// (release), and a block of k_raster_fast that loads this frame's number (acquire)
+// sees all that was visible to that thread: the list, the counters and the cleared
+// keys. An older number (the store has not arrived, or another kernel was queued
+// between the two) takes the wait, after which the same holds. A frame's number is
+// never 0 and differs from those before it in the same scratch; a replayed graph
+// repeats its number, but its kernels run one after the other.
+__device__ __forceinline__ void give_list(const Scratch& s, uint32_t front) {
+    asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(s.counters + C_LIST),
+                 "l"((unsigned long long)s.frame << 32 | front)
+                 : "memory");
+}
+__device__ __forceinline__ uint32_t take_list(const Scratch& s) {
+    __shared__ unsigned long long given;
+    if (threadIdx.x == 0) {
+        unsigned long long w;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(s.counters + C_LIST) : "memory");
+        given = w;
+    }
+    __syncthreads();
+    uint32_t front = (uint32_t)given;
+    if ((uint32_t)(given >> 32) != s.frame) {
+        uint32_t back;
+        wait_for_previous();
+        entry_counts(s, front, back);
+    }
+    return front;
+}
+
 // One segment for one view at its precision k on the general path.
 template <bool STREAM>
 __device__ __forceinline__ uint32_t segment_k(const CloudView& c, const ViewConst& vc,
@@ -1557,8 +1589,8 @@ __device__ __forceinline__ void flush_atomics(const Scratch& s, uint32_t view, u
 // One view per launch: two kernels, so that neither path's registers burden the
 // other. The certified entries (the draw list's front) go to k_raster_fast, the
 // others (its back) to k_raster_general, launched just before it. The fast
-// kernel starts as soon as the general one's blocks have started
-// (programmatic launch): both only read what the cull pass wrote and update the
+// kernel starts as soon as the general one's blocks have started and the list is
+// handed over (take_list): both only read what the first pass wrote and update the
 // view by atomics, so they may run side by side. In one kernel at 48 registers
 // the general path spilled (a 100M-point fly-through frame's raster pass took
 // 99 us, 74 us with two kernels); at 64 registers both paths fit, but the fast
@@ -1571,8 +1603,7 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
                                                                Scratch s) {
     start_next();
     const uint32_t lane = threadIdx.x & 31;
-    uint32_t n_entries, n_back;
-    entry_counts(s, n_entries, n_back);
+    const uint32_t n_entries = take_list(s);
     uint32_t n_atom = 0;
     for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
         const DrawEntry e = s.entries[i];
@@ -1592,12 +1623,20 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
 
 __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView c, ViewTable vt,
                                                                   Scratch s) {
-    // the fast kernel may start once the draw list is there
     wait_for_previous();
-    start_next();
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_front, n_entries;
-    entry_counts(s, n_front, n_entries);
+    if (blockIdx.x == 0) {
+        // the fast kernel starts when every block has come past start_next, by
+        // which time the list is on its way
+        entry_counts(s, n_front, n_entries);
+        if (threadIdx.x == 0) give_list(s, n_front);
+        __syncthreads();
+        start_next();
+    } else {
+        start_next();
+        entry_counts(s, n_front, n_entries);
+    }
     const ViewConst vc = make_view_const(vt.v[0]);
     uint32_t n_atom = 0;
     for (uint32_t i = first_entry(n_entries); i < n_entries;
@@ -2139,7 +2178,7 @@ __device__ __forceinline__ void publish_frame(uint32_t nviews, uint32_t view_bas
         s.stats[(uint64_t)view_base * S_COUNT + i] = s.acc[i];
         s.acc[i] = 0ull;
     }
-    if (threadIdx.x < C_COUNT && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
+    if (threadIdx.x < C_LIST && threadIdx.x != C_ERROR && threadIdx.x != C_ERRINFO)
         s.counters[threadIdx.x] = 0u;
 }
 
