@@ -281,8 +281,8 @@ pc_status pc_render(pc_ctx* ctx, pc_cloud cloud, const pc_view* views, uint32_t 
  * device_error (host memory, two words, may be NULL): the call ends by copying
  * the kernels' error flag and its value there, stream-ordered; once the stream
  * has reached that point, a nonzero first word means the image is not valid
- * (a batch outside the point buffers, batches that overlap so that the draw
- * list overflows). Pinned memory keeps the copy asynchronous; pageable memory
+ * (a batch outside the point buffers; batches that overlap so that the draw
+ * list overflows, of which what fits is drawn). Pinned memory keeps the copy asynchronous; pageable memory
  * makes the call wait for the stream and cannot be used during a capture.
  * The first call on a device looks up that
  * array's device address (a runtime call, no allocation) and keeps it for the

@@ -390,14 +390,22 @@ __device__ void append_batches(CullShared& sh, uint32_t first, uint32_t n, const
                                          warp_sum(kl >= 2u ? count : 0u) + warp_sum(kl == 3u ? count : 0u);
         if (lane == 0 && words) atomicAdd(&sh.words, words);
         base = __shfl_sync(FULL, base, 31);
-        // both lists together fit the buffer up to this warp's reservation, or none
-        // of its entries is written (later reservations do not fit then either)
-        const uint64_t end = (base >> 32) + (uint32_t)base + (total >> 32) + (uint32_t)total;
-        if (end > s.capacity) {
-            if (nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)end);
-            // the counts must not come round to a sum that looks as if it fitted
-            if (lane == 31) atomicOr(&s.counters[C_GENERAL], 0x80000000u);
-            nseg = 0;
+        // Past the end of the buffer (batches that overlap in caller-provided buffers)
+        // the reservation keeps what fits, in its order, and gives the rest back: only
+        // the one that crosses the end keeps a part, those after it nothing, and the
+        // counts end at what was written.
+        const uint64_t used = (base >> 32) + (uint32_t)base;
+        const uint64_t room = used < s.capacity ? s.capacity - used : 0ull;
+        if ((total >> 32) + (uint32_t)total > room) {
+            const uint64_t before = (incl >> 32) + (uint32_t)incl - nseg;
+            const uint32_t fit = before < room ? (uint32_t)min((uint64_t)nseg, room - before) : 0u;
+            if (fit < nseg) raise_error(s, E_ENTRY_RANGE, (uint32_t)(used + before + fit));
+            const uint32_t front = __reduce_add_sync(FULL, general ? 0u : nseg - fit);
+            const uint32_t back = __reduce_add_sync(FULL, general ? nseg - fit : 0u);
+            if (lane == 0)
+                atomicAdd(reinterpret_cast<unsigned long long*>(s.counters + C_ENTRIES),
+                          0ull - ((unsigned long long)back << 32 | front));
+            nseg = fit;
         }
         if (i < n) {
             const unsigned long long at = base + incl - own;
@@ -1530,11 +1538,11 @@ __device__ __forceinline__ uint32_t fan_out(uint32_t i, uint32_t n) {
     return i < rounds * kFan ? (i % kFan) * rounds + i / kFan : i;
 }
 
-// Lengths of the draw list's two parts; none when they overflowed the buffer.
+// Lengths of the draw list's two parts (together within the buffer, see
+// append_batches; no entry outside it is read all the same).
 __device__ __forceinline__ void entry_counts(const Scratch& s, uint32_t& front, uint32_t& back) {
-    front = s.counters[C_ENTRIES];
-    back = s.counters[C_GENERAL];
-    if ((uint64_t)front + back > s.capacity) front = back = 0;
+    front = (uint32_t)min((uint64_t)s.counters[C_ENTRIES], s.capacity);
+    back = (uint32_t)min((uint64_t)s.counters[C_GENERAL], s.capacity - front);
 }
 
 // The draw list's way from k_raster_general to k_raster_fast, which runs beside it
