@@ -76,6 +76,32 @@ Slot::~Slot() {
     cudaFree(host_rgba);
 }
 
+// True while the stream is being captured: work on it is then recorded and has not
+// run (also taken for true when the stream cannot be asked).
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
+
+// Zero, in stream order, of what a frame's last pass leaves at zero (the sums, and the
+// counters but the error words), or of the whole allocation.
+static cudaError_t clear_scratch(const Slot& s, bool all) {
+    const size_t sums = kMaxViewsPerLaunch * S_COUNT;
+    if (all)
+        return cudaMemsetAsync(s.scratch.counters, 0,
+                               sizeof(uint32_t) * C_COUNT +
+                                   sizeof(unsigned long long) * (sums + kMaxViewsPerRender * S_COUNT),
+                               s.stream);
+    cudaError_t e = cudaMemsetAsync(s.scratch.acc, 0, sizeof(unsigned long long) * sums, s.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(s.scratch.counters, 0, sizeof(uint32_t) * C_ERROR, s.stream);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(s.scratch.counters + C_ERRINFO + 1, 0,
+                            sizeof(uint32_t) * (C_LIST - C_ERRINFO - 1), s.stream);
+    return e;
+}
+
 pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
     // counters, sums and statistics are one allocation, the others each on its
     // own, so a failed allocation is retried by the next call
@@ -86,21 +112,14 @@ pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
         if (e != cudaSuccess) return cuda_fail(e, "scratch counters");
         s.scratch.counters = reinterpret_cast<uint32_t*>(p);
         s.scratch.acc = p + C_COUNT / 2;
-        s.scratch.stats = s.scratch.acc + kMaxViewsPerLaunch * S_COUNT;
-        cudaMemsetAsync(p, 0, words * sizeof(unsigned long long), s.stream);
+        s.unclean = Unclean::kAll;
     }
-    if (s.unclean) {
-        // a frame whose launches failed part-way: its last pass did not leave
-        // the counters (the error words apart) and sums at zero
-        cudaError_t e = cudaMemsetAsync(s.scratch.acc, 0,
-                                        sizeof(unsigned long long) * kMaxViewsPerLaunch * S_COUNT, s.stream);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(s.scratch.counters, 0, sizeof(uint32_t) * C_ERROR, s.stream);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(s.scratch.counters + C_ERRINFO + 1, 0,
-                                sizeof(uint32_t) * (C_LIST - C_ERRINFO - 1), s.stream);
+    if (s.unclean != Unclean::kNo) {
+        const cudaError_t e = clear_scratch(s, s.unclean == Unclean::kAll);
         if (e != cudaSuccess) return cuda_fail(e, "scratch reset");
-        s.unclean = false;
+        s.scratch.stats = s.scratch.acc + kMaxViewsPerLaunch * S_COUNT;   // to be read from now on
+        // a recorded clear is the graph's, not the next queued frame's
+        if (!capturing(s.stream)) s.unclean = Unclean::kNo;
     }
     if (entries > s.scratch.capacity) {
         cudaStreamSynchronize(s.stream);
@@ -370,7 +389,15 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
     rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, fo);
-    if (rc != PC_OK) slot->unclean = true;
+    if (rc != PC_OK && !graph) {
+        // The last pass, which leaves the scratch at zero, is missing: clear it behind
+        // what was launched, for whatever uses it next (a replayed graph passes no
+        // call of the library). While a caller captures, that part and its clearing
+        // are the graph's and the scratch is as it was.
+        if (clear_scratch(*slot, false) != cudaSuccess && cs == cudaStreamCaptureStatusNone &&
+            slot->unclean == Unclean::kNo)
+            slot->unclean = Unclean::kFrame;
+    }
     if (graph) {
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(st, &g);

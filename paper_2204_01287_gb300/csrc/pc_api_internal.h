@@ -50,6 +50,12 @@ struct Cloud {
     ~Cloud() { free_device(); }
 };
 
+// What a stream's scratch needs before its next frame, which takes its counters and
+// sums to be zero: nothing (every frame leaves them so); their clearing, since a frame's
+// launches failed part-way and so did the clearing behind them; or that of the
+// whole, new allocation.
+enum class Unclean { kNo, kFrame, kAll };
+
 // Scratch and library-owned framebuffers of one stream.
 struct Slot {
     cudaStream_t stream = nullptr;
@@ -61,7 +67,7 @@ struct Slot {
     uint64_t* host_vis = nullptr;     // pc_render_host framebuffers
     uint32_t* host_rgba = nullptr;
     uint64_t host_pixels = 0;
-    bool unclean = false;           // a frame's launches failed part-way (see ensure_capacity)
+    Unclean unclean = Unclean::kNo;
     uint32_t last_nviews = 0;
     uint64_t last_total_batches = 0;
     std::map<uint64_t, cudaGraphExec_t> graphs;   // replayable frames by launch layout
