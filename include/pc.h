@@ -66,7 +66,9 @@ typedef struct {
     float    precision_px;        /* T: k = 1 if the projected batch extent < T px,
                                      2 if < 1024 T, else 3 (default 512 = 0.5 px per cell
                                      of 1024; the paper's 500 is selectable, Sec. 3.3) */
-    uint32_t encoder_threads;     /* host encoder threads, 0 = all cores */
+    uint32_t encoder_threads;     /* host encoder threads, 0 = all cores (pc_upload_cloud
+                                     encodes on the device and uses them only where that
+                                     has no room) */
     uint32_t flags;               /* PC_CFG_* */
     uint64_t serve_pool_bytes;    /* device memory for library-owned serving framebuffers
                                      (default 2 GiB) */
@@ -127,9 +129,9 @@ pc_status pc_encode(const float* xyz, const uint32_t* rgba, uint64_t n,
 /* Encode host points (with the bits of pc_encode; batch size and
  * PC_CFG_KEEP_ORDER from the context's config) into a cloud in device memory owned
  * by the library. The encoder runs on the device, with scratch memory of 40 bytes
- * a point during the call, or on the host where the device has no room for
- * it. Synchronous. xyz and rgba are read only during the call. *out receives a
- * cloud handle. */
+ * a point during the call (beside the cloud's 16), or on the host where the device
+ * has no room for it; PC_ENOMEM when the cloud itself does not fit. Synchronous.
+ * xyz and rgba are read only during the call. *out receives a cloud handle. */
 pc_status pc_upload_cloud(pc_ctx* ctx, const float* xyz, const uint32_t* rgba,
                           uint64_t n, pc_cloud* out);
 

@@ -561,32 +561,49 @@ pc_cloud Ctx::register_cloud(const std::shared_ptr<Cloud>& cl) {
 }
 
 // A cloud's device buffers for n points in nbatches batches (contents unset but
-// for the words past n, which are 0).
-static pc_status allocate_cloud(Ctx& ctx, uint64_t n, uint64_t nbatches, uint64_t entries,
-                                std::shared_ptr<Cloud>& out) {
+// for the words past n, which are 0). Leaves no message, but the error in e: without
+// room (PC_ENOMEM) the caller may try again.
+static pc_status allocate_cloud(uint64_t n, uint64_t nbatches, uint64_t entries,
+                                std::shared_ptr<Cloud>& out, cudaError_t& e) {
     auto cl = std::make_shared<Cloud>();
     cl->n_points = n;
     cl->n_batches = nbatches;
     cl->n_entries = std::max<uint64_t>(entries, 1);
     const uint64_t npad = ((n + 3) & ~3ull) + 4;   // 16-byte groups never run past the end
     uint32_t** bufs[4] = {&cl->w1, &cl->w2, &cl->w3, &cl->color};
-    cudaError_t e = cudaMalloc(&cl->batches, std::max<uint64_t>(1, nbatches) * sizeof(pc_batch));
+    e = cudaMalloc(&cl->batches, std::max<uint64_t>(1, nbatches) * sizeof(pc_batch));
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) e = cudaMalloc(bufs[i], npad * sizeof(uint32_t));
-    if (e != cudaSuccess) {
-        cl->free_device();
-        ctx.fail_msg("cloud allocation (%llu points): %s", (unsigned long long)n,
-                     cudaGetErrorString(e));
-        return PC_ENOMEM;
-    }
+    const bool room = e == cudaSuccess;
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
         e = cudaMemset(*bufs[i] + n, 0, (npad - n) * sizeof(uint32_t));
     if (e != cudaSuccess) {
+        cudaGetLastError();   // not the next launch's error
         cl->free_device();
-        return ctx.cuda_fail(e, "cloud upload");
+        return room ? PC_ECUDA : PC_ENOMEM;
     }
     cl->device_bytes = 4 * npad * sizeof(uint32_t) + nbatches * sizeof(pc_batch);
     out = cl;
     return PC_OK;
+}
+
+// The message of allocate_cloud's status rc.
+static pc_status allocation_failed(Ctx& ctx, pc_status rc, cudaError_t e, uint64_t n) {
+    if (rc == PC_ECUDA) return ctx.cuda_fail(e, "cloud upload");
+    ctx.fail_msg("cloud allocation (%llu points): %s", (unsigned long long)n, cudaGetErrorString(e));
+    return rc;
+}
+
+// Copies an encoded cloud into its device buffers.
+static cudaError_t copy_encoded(Cloud& cl, const pc_batch* batches, const uint32_t* w1, const uint32_t* w2,
+                                const uint32_t* w3, const uint32_t* color) {
+    uint32_t* bufs[4] = {cl.w1, cl.w2, cl.w3, cl.color};
+    const uint32_t* src[4] = {w1, w2, w3, color};
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 4 && e == cudaSuccess && cl.n_points; ++i)
+        e = cudaMemcpy(bufs[i], src[i], cl.n_points * sizeof(uint32_t), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && cl.n_batches)
+        e = cudaMemcpy(cl.batches, batches, cl.n_batches * sizeof(pc_batch), cudaMemcpyHostToDevice);
+    return e;
 }
 
 // Copy an encoded cloud to library-owned device memory (no handle yet).
@@ -610,28 +627,44 @@ pc_status upload_encoded_internal(Ctx& c, const pc_batch* batches, uint64_t nbat
     }
     cudaSetDevice(ctx->device);
     std::shared_ptr<Cloud> cl;
-    pc_status rc = allocate_cloud(c, n, nbatches, entries, cl);
-    if (rc != PC_OK) return rc;
-    uint32_t* bufs[4] = {cl->w1, cl->w2, cl->w3, cl->color};
-    const uint32_t* src[4] = {w1, w2, w3, color};
     cudaError_t e = cudaSuccess;
-    for (int i = 0; i < 4 && e == cudaSuccess && n; ++i)
-        e = cudaMemcpy(bufs[i], src[i], n * sizeof(uint32_t), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && nbatches)
-        e = cudaMemcpy(cl->batches, batches, nbatches * sizeof(pc_batch), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-        cl->free_device();
-        return ctx->cuda_fail(e, "cloud upload");
-    }
+    const pc_status rc = allocate_cloud(n, nbatches, entries, cl, e);
+    if (rc != PC_OK) return allocation_failed(c, rc, e, n);
+    e = copy_encoded(*cl, batches, w1, w2, w3, color);
+    if (e != cudaSuccess) return ctx->cuda_fail(e, "cloud upload");
     out = cl;
     return PC_OK;
 }
 
-// Encode raw points on the device into a new cloud (no handle yet), with the same
-// bits as the host encoder. PC_ENOMEM without a message: the device has no room
-// for the encoder's scratch (40 bytes a point) beside the cloud.
+// Encodes raw points on the host into a new cloud's device buffers.
+static pc_status encode_on_host(Ctx& c, const float* xyz, const uint32_t* rgba, Cloud& cl) {
+    std::vector<pc_batch> batches;
+    std::vector<uint32_t> words[4];   // three of coordinates, the colours
+    try {
+        batches.resize(cl.n_batches);
+        for (auto& w : words) w.resize(cl.n_points);
+    } catch (...) {
+        c.fail_msg("host memory for encoding %llu points", (unsigned long long)cl.n_points);
+        return PC_ENOMEM;
+    }
+    const uint32_t eflags = (c.cfg.flags & PC_CFG_KEEP_ORDER) ? PC_ENCODE_KEEP_ORDER : 0u;
+    const pc_status rc =
+        pc_encode(xyz, rgba, cl.n_points, c.cfg.batch_size, c.cfg.encoder_threads, eflags, batches.data(),
+                  words[0].data(), words[1].data(), words[2].data(), words[3].data(), nullptr);
+    if (rc != PC_OK) {
+        c.fail_msg("encoder failed: %s", pc_strerror(rc));
+        return rc;
+    }
+    const cudaError_t e = copy_encoded(cl, batches.data(), words[0].data(), words[1].data(), words[2].data(),
+                                       words[3].data());
+    return e == cudaSuccess ? PC_OK : c.cuda_fail(e, "cloud upload");
+}
+
+// Encode raw points (n > 0) into a new cloud (no handle yet): on the device, or, when
+// it has no room for the encoder's scratch (40 bytes a point) beside the cloud, on
+// the host with the same bits.
 // The host encoder took 32 ms for 4M points on 16 cores, half of it in page faults
-// of its arrays; this takes 1.6 ms: the copy of 64 MB 0.4, the kernels 0.8, the
+// of its arrays; the device takes 1.6 ms: the copy of 64 MB 0.4, the kernels 0.8, the
 // allocations the rest.
 static pc_status upload_points(Ctx& c, const float* xyz, const uint32_t* rgba, uint64_t n,
                                std::shared_ptr<Cloud>& out) {
@@ -642,30 +675,34 @@ static pc_status upload_points(Ctx& c, const float* xyz, const uint32_t* rgba, u
                              (last + kMinSegmentPoints - 1) / kMinSegmentPoints;
     void* scratch = nullptr;
     if (cudaMalloc(&scratch, encode_device_scratch(n, rgba != nullptr, keep)) != cudaSuccess) {
-        cudaGetLastError();   // the host encoder takes over
-        return PC_ENOMEM;
+        cudaGetLastError();
+        scratch = nullptr;
     }
     std::shared_ptr<Cloud> cl;
-    pc_status rc = allocate_cloud(c, n, nb, entries, cl);
-    if (rc == PC_ENOMEM) {   // perhaps without the scratch
-        cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    pc_status rc = allocate_cloud(n, nb, entries, cl, e);
+    if (rc == PC_ENOMEM && scratch) {
         cudaFree(scratch);
-        return rc;
+        scratch = nullptr;
+        rc = allocate_cloud(n, nb, entries, cl, e);
     }
-    bool finite = false;
-    if (rc == PC_OK) {
-        const cudaError_t e = encode_device(xyz, rgba, n, bs, keep, scratch, cl->batches, cl->w1,
-                                            cl->w2, cl->w3, cl->color, cudaStreamLegacy, &finite);
-        if (e != cudaSuccess) rc = c.cuda_fail(e, "cloud encoding");
+    if (rc != PC_OK) rc = allocation_failed(c, rc, e, n);
+    if (rc == PC_OK && !scratch) {
+        rc = encode_on_host(c, xyz, rgba, *cl);
+    } else if (rc == PC_OK) {
+        bool finite = false;
+        e = encode_device(xyz, rgba, n, bs, keep, scratch, cl->batches, cl->w1, cl->w2, cl->w3, cl->color,
+                          cudaStreamLegacy, &finite);
+        if (e != cudaSuccess) {
+            rc = c.cuda_fail(e, "cloud encoding");
+        } else if (!finite) {
+            c.fail_msg("encoder failed: %s", pc_strerror(PC_EINVAL));
+            rc = PC_EINVAL;
+        }
     }
     cudaFree(scratch);
-    if (rc != PC_OK) return rc;
-    if (!finite) {
-        c.fail_msg("encoder failed: %s", pc_strerror(PC_EINVAL));
-        return PC_EINVAL;
-    }
-    out = cl;
-    return PC_OK;
+    if (rc == PC_OK) out = cl;
+    return rc;
 }
 
 }  // namespace pcr
@@ -696,37 +733,13 @@ pc_status pc_upload_cloud(pc_ctx* h, const float* xyz, const uint32_t* rgba, uin
         ctx->fail_msg("cloud too large: %llu points", (unsigned long long)n);
         return PC_EINVAL;
     }
+    std::shared_ptr<Cloud> cl;
     cudaSetDevice(ctx->device);
-    if (n) {
-        std::shared_ptr<Cloud> cl;
-        const pc_status rc = upload_points(*ctx, xyz, rgba, n, cl);
-        if (rc == PC_OK) *out = ctx->register_cloud(cl);
-        if (rc != PC_ENOMEM) return rc;
-    }
-    // no points, or no room on the device for the encoder: encode on the host
-    const uint32_t bs = ctx->cfg.batch_size;
-    const uint64_t nb = (n + bs - 1) / bs;
-    std::vector<pc_batch> batches;
-    std::vector<uint32_t> w1, w2, w3, color;
-    try {
-        batches.resize(nb);
-        w1.resize(n);
-        w2.resize(n);
-        w3.resize(n);
-        color.resize(n);
-    } catch (...) {
-        ctx->fail_msg("host memory for encoding %llu points", (unsigned long long)n);
-        return PC_ENOMEM;
-    }
-    const uint32_t eflags = (ctx->cfg.flags & PC_CFG_KEEP_ORDER) ? PC_ENCODE_KEEP_ORDER : 0u;
-    pc_status rc = pc_encode(xyz, rgba, n, bs, ctx->cfg.encoder_threads, eflags, batches.data(),
-                             w1.data(), w2.data(), w3.data(), color.data(), nullptr);
-    if (rc != PC_OK) {
-        ctx->fail_msg("encoder failed: %s", pc_strerror(rc));
-        return rc;
-    }
-    return pc_upload_encoded(h, batches.data(), nb, w1.data(), w2.data(), w3.data(),
-                             color.data(), n, out);
+    const pc_status rc =
+        n ? upload_points(*ctx, xyz, rgba, n, cl)
+          : upload_encoded_internal(*ctx, nullptr, 0, nullptr, nullptr, nullptr, nullptr, 0, cl);
+    if (rc == PC_OK) *out = ctx->register_cloud(cl);
+    return rc;
 }
 
 pc_status pc_cloud_get_info(pc_ctx* h, pc_cloud cloud, pc_cloud_info* info) {

@@ -6,6 +6,7 @@
 // stream runs at once, or is recorded while the stream is captured. A frame's first
 // pass notes whether its counters and sums start from zero, its last one leaves
 // them so; what lies between dirties them.
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -26,7 +27,7 @@ struct CUgraphExec_st { Ops ops; };
 
 static Ops* g_recording = nullptr;        // the captured stream's work
 static std::map<std::string, int> g_fail; // call -> calls until one fails (1: the next)
-static int g_dirty = 0, g_frames = 0, g_instantiated = 0;
+static int g_dirty = 0, g_frames = 0, g_instantiated = 0, g_encoded = 0;
 static size_t g_room = ~(size_t)0, g_used = 0;   // bytes the "device" has, and lent
 static std::map<void*, size_t> g_blocks;
 
@@ -176,6 +177,7 @@ uint64_t encode_device_scratch(uint64_t n, bool, bool) { return 40 * n; }
 cudaError_t encode_device(const float* xyz, const uint32_t* rgba, uint64_t n, uint32_t batch_size, bool keep_order,
                           void*, pc_batch* batches, uint32_t* w1, uint32_t* w2, uint32_t* w3, uint32_t* color,
                           cudaStream_t, bool* finite) {
+    ++g_encoded;
     *finite = encode_host(xyz, rgba, n, batch_size, 1, keep_order, batches, w1, w2, w3, color, nullptr) == PC_OK;
     return cudaSuccess;
 }
@@ -311,6 +313,53 @@ static void first_frame_captured() {
     cudaGraphExecDestroy(e);
 }
 
+// pc_upload_cloud where the encoder's scratch does not fit beside the cloud: the host
+// encodes, with the same bits and no message left; where the cloud does not fit
+// either, the call fails before any encoding.
+static void upload_without_room() {
+    const uint64_t n = 10000, cloud = 16 * n, scratch = 40 * n;
+    World w(0, n);
+    pc_cloud_info info;
+    CHECK(pc_cloud_get_info(w.ctx, w.cloud, &info) == PC_OK);
+    auto bytes = [&](pc_cloud c) {
+        std::vector<pc_batch> b(info.n_batches);
+        std::vector<uint32_t> words(4 * n);
+        CHECK(pc_cloud_download(w.ctx, c, b.data(), &words[0], &words[n], &words[2 * n], &words[3 * n]) == PC_OK);
+        std::string s((const char*)b.data(), b.size() * sizeof(pc_batch));
+        return s + std::string((const char*)words.data(), words.size() * 4);
+    };
+    const std::string expect = bytes(w.cloud);
+    const size_t used = g_used;
+    // room for the scratch and the cloud, for either but not both, for the cloud alone
+    for (size_t room : {scratch + 2 * cloud, scratch + cloud / 2, 2 * cloud}) {
+        const int before = g_encoded;
+        g_room = used + room;
+        pc_cloud c = 0;
+        CHECK(pc_upload_cloud(w.ctx, w.xyz.data(), nullptr, n, &c) == PC_OK);
+        CHECK(g_encoded - before == (room == scratch + 2 * cloud));
+        CHECK(bytes(c) == expect);
+        CHECK(std::string(pc_last_error(w.ctx)).empty());
+        CHECK(pc_release_cloud(w.ctx, c) == PC_OK);
+        CHECK(g_used == used);
+    }
+    // room for a part of the cloud only: refused at once, all given back
+    pc_cloud c = 0;
+    g_room = used + cloud / 2;
+    const uint64_t encoded = g_encoded;
+    std::vector<float> bad(3 * n, 0.0f);
+    bad[7] = INFINITY;   // the host encoder would say so
+    CHECK(pc_upload_cloud(w.ctx, bad.data(), nullptr, n, &c) == PC_ENOMEM);
+    CHECK(g_encoded == (int)encoded && g_used == used && c == 0);
+    CHECK(std::string(pc_last_error(w.ctx)).find("cloud allocation") != std::string::npos);
+    // what the device encoder refuses leaves nothing behind either
+    g_room = ~(size_t)0;
+    CHECK(pc_upload_cloud(w.ctx, bad.data(), nullptr, n, &c) == PC_EINVAL);
+    CHECK(g_used == used && c == 0);
+    // the empty cloud
+    CHECK(pc_upload_cloud(w.ctx, nullptr, nullptr, 0, &c) == PC_OK);
+    CHECK(pc_cloud_get_info(w.ctx, c, &info) == PC_OK && info.n_points == 0 && info.n_batches == 0);
+}
+
 static const std::map<std::string, void (*)()>& scenarios() {
     static const std::map<std::string, void (*)()> all = {
         {"failed_frame", failed_frame},
@@ -320,6 +369,7 @@ static const std::map<std::string, void (*)()>& scenarios() {
         {"failed_clearing_is_tried_again", failed_clearing_is_tried_again},
         {"first_clearing_fails", first_clearing_fails},
         {"first_frame_captured", first_frame_captured},
+        {"upload_without_room", upload_without_room},
     };
     return all;
 }
