@@ -229,10 +229,11 @@ uint32_t Ctx::views_per_launch(const Cloud& cl) const {
     return std::max<uint32_t>(1, std::min<uint32_t>(v, kMaxViewsPerLaunch));
 }
 
-// The kernels of one frame: per launch group, clear / cull / raster / resolve.
+// The kernels of one frame: per launch group, clear and cull / raster / shade /
+// resolve. *kernels: how many.
 pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                             const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
-                            uint32_t maxv, bool timing, const FrameOpts& fo) {
+                            uint32_t maxv, bool timing, const FrameOpts& fo, uint32_t* kernels) {
     CloudView cv = cl.view();
     if (fo.first || fo.count < cl.n_batches) {
         // a shard: the kernels see only the batches of the range (their point
@@ -286,7 +287,7 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
             e = launch_resolve(cv, vt, base, slot->scratch, false, st, &resolve_kernels);
             if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
             if (fe) cudaEventRecord(fe->ev[5], st);
-            launches += resolve_kernels;
+            *kernels += resolve_kernels;
             continue;
         }
         if (fe) cudaEventRecord(fe->ev[1], st);   // the clear runs beside the culling
@@ -295,7 +296,7 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         if (cl.is_lod) {
             e = launch_lod_append(cv, vt, slot->scratch, st);
             if (e != cudaSuccess) return cuda_fail(e, "LOD selection launch");
-            launches += 1;
+            *kernels += 1;
         }
         if (fe) cudaEventRecord(fe->ev[2], st);
         int raster_kernels = 0;
@@ -307,14 +308,14 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
             int nk = 0;
             e = launch_shade(cv, vt, slot->scratch, shape, st, &nk);
             if (e != cudaSuccess) return cuda_fail(e, "shading launch");
-            launches += nk;
+            *kernels += nk;
         }
         if (fe) cudaEventRecord(fe->ev[4], st);
         int resolve_kernels = 0;
         e = launch_resolve(cv, vt, base, slot->scratch, true, st, &resolve_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "resolve launch");
         if (fe) cudaEventRecord(fe->ev[5], st);
-        launches += 1 + raster_kernels + resolve_kernels;
+        *kernels += 1 + raster_kernels + resolve_kernels;
         raster_launches += 1;
     }
     return PC_OK;
@@ -388,7 +389,9 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
-    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, fo);
+    uint32_t kernels = 0;
+    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, fo, &kernels);
+    launches += kernels;
     if (rc != PC_OK && !graph) {
         // The last pass, which leaves the scratch at zero, is missing: clear it behind
         // what was launched, for whatever uses it next (a replayed graph passes no
@@ -406,10 +409,13 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
             return rc;
         }
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
-        uint64_t shaded = 0;   // the views with a colour pass change the launch layout
+        // one instantiated graph per launch layout, so that programs which alternate
+        // between layouts (plain and dilated views, with and without a colour pass) keep
+        // updating: the number of kernels tells the layouts of one view count apart
+        uint64_t shaded = 0;
         for (uint32_t v = 0; v < nviews; ++v) shaded |= (uint64_t)(hqs_mode(views[v].flags) != 0);
         const uint64_t key = ((uint64_t)nviews << 8) | maxv | ((uint64_t)cl.is_lod << 40) |
-                             (shaded << 41) | ((uint64_t)fo.resolve_only << 42);
+                             (shaded << 41) | ((uint64_t)fo.resolve_only << 42) | ((uint64_t)kernels << 43);
         cudaGraphExec_t& exec = slot->graphs[key];
         if (exec) {
             cudaGraphExecUpdateResultInfo info;

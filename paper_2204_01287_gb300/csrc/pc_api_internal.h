@@ -123,7 +123,7 @@ struct Ctx {
     void set_tune(Cloud& cl, uint32_t nviews, const Tune& t);
     pc_status launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                            const pc_framebuffer* fbs, cudaStream_t st, Slot* slot, uint32_t maxv,
-                           bool timing, const FrameOpts& fo);
+                           bool timing, const FrameOpts& fo, uint32_t* kernels);
     pc_status render(const Cloud& cl, const pc_view* views, uint32_t nviews,
                      const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
                      const FrameOpts& fo = FrameOpts());

@@ -360,6 +360,21 @@ static void upload_without_room() {
     CHECK(pc_cloud_get_info(w.ctx, c, &info) == PC_OK && info.n_points == 0 && info.n_batches == 0);
 }
 
+// PC_CFG_GRAPHS: a program that alternates between launch layouts of one view count
+// instantiates one graph for each and then only updates.
+static void graphs_of_alternating_layouts() {
+    World w(PC_CFG_GRAPHS);
+    const std::vector<std::vector<uint32_t>> layouts = {
+        {0u, 0u}, {0u, PC_VIEW_DILATE}, {PC_VIEW_DILATE, PC_VIEW_DILATE}, {PC_VIEW_HQS, 0u},
+        {PC_VIEW_HQS_PACKED, 0u}, {PC_VIEW_HQS_PACKED, PC_VIEW_DILATE}};
+    for (const auto& l : layouts) CHECK(w.frame(l) == PC_OK);
+    const int made = g_instantiated;
+    CHECK(made <= (int)layouts.size());
+    for (int i = 0; i < 3; ++i)
+        for (const auto& l : layouts) CHECK(w.frame(l) == PC_OK);
+    CHECK(g_instantiated == made && g_dirty == 0);
+}
+
 static const std::map<std::string, void (*)()>& scenarios() {
     static const std::map<std::string, void (*)()> all = {
         {"failed_frame", failed_frame},
@@ -370,6 +385,7 @@ static const std::map<std::string, void (*)()>& scenarios() {
         {"first_clearing_fails", first_clearing_fails},
         {"first_frame_captured", first_frame_captured},
         {"upload_without_room", upload_without_room},
+        {"graphs_of_alternating_layouts", graphs_of_alternating_layouts},
     };
     return all;
 }
