@@ -2368,19 +2368,28 @@ __device__ __forceinline__ void dilate_pixels(DilateTile& t, const uint32_t (&ra
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(256) k_resolve_dilated(CloudView c, ViewTable vt, uint32_t view_base,
-                                                       Scratch s, bool publish) {
+// The dilating resolve's grid: the tiles of the views that dilate into an image and no
+// others, view after view (end: where each one's end). With the largest view's number of
+// tiles for every view, one dilated view of 2016x2240 beside 31 views of 64x48 took
+// 215 us in both resolves, 50 us this way. Eight blocks per SM (32 registers): at the
+// 40 registers that the search for the view takes otherwise, a headset frame took 10 us more.
+struct TileGrid {
+    uint32_t end[kMaxViewsPerLaunch];
+};
+
+__global__ void __launch_bounds__(256, 8) k_resolve_dilated(CloudView c, ViewTable vt, TileGrid grid,
+                                                       uint32_t view_base, Scratch s, bool publish) {
     start_next();
     wait_for_previous();
-    if (publish && blockIdx.y == 0 && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
-    const ViewParams& vp = vt.v[blockIdx.y];
-    if (!vp.rgba || !(vp.flags & PC_VIEW_DILATE)) return;
+    if (publish && blockIdx.x == 0) publish_frame(vt.n, view_base, s);
+    uint32_t v = 0, first = 0;
+    while (blockIdx.x >= grid.end[v]) first = grid.end[v++];
+    const uint32_t tile = blockIdx.x - first;
+    const ViewParams vp = vt.v[v];   // once: v is not a constant of the block to the compiler
     const int W = (int)vp.width, H = (int)vp.height;
-    const int tiles_x = (W + kTile - 1) / kTile, tiles_y = (H + kTile - 1) / kTile;
-    if (blockIdx.x >= (uint32_t)(tiles_x * tiles_y)) return;
+    const uint32_t tiles_x = (vp.width + kTile - 1) / kTile;
     __shared__ DilateTile t;
-    const int ox = (int)(blockIdx.x % (uint32_t)tiles_x) * kTile;
-    const int oy = (int)(blockIdx.x / (uint32_t)tiles_x) * kTile;
+    const int ox = (int)(tile % tiles_x) * kTile, oy = (int)(tile / tiles_x) * kTile;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     for (int y = ty; y < kTileIn; y += 8)
         for (int x = tx; x < kTileIn; x += 32) {
@@ -2591,22 +2600,26 @@ cudaError_t launch_merge_min(uint64_t* dst, const uint64_t* src, uint64_t n, cud
 
 cudaError_t launch_resolve(const CloudView& c, const ViewTable& vt, uint32_t view_base, Scratch s,
                            bool publish, cudaStream_t st, int* launched) {
-    uint64_t maxpix = 0, maxtiles = 0;
+    uint64_t maxpix = 0;
+    TileGrid grid{};
+    uint32_t tiles = 0;   // at most 32 views of 512 x 512 tiles
     bool plain = false, shaded = false;
     for (uint32_t v = 0; v < vt.n; ++v) {
-        const uint64_t w = vt.v[v].width, h = vt.v[v].height;
-        if (vt.v[v].flags & PC_VIEW_DILATE)
-            maxtiles = max(maxtiles, ((w + kTile - 1) / kTile) * ((h + kTile - 1) / kTile));
-        else
-            plain = true;
+        const bool dilated = vt.v[v].flags & PC_VIEW_DILATE;
+        if (dilated && vt.v[v].rgba)
+            tiles += ((vt.v[v].width + kTile - 1) / kTile) * ((vt.v[v].height + kTile - 1) / kTile);
+        grid.end[v] = tiles;
+        if (dilated) continue;
+        plain = true;
         shaded |= vt.v[v].accum != nullptr;
-        maxpix = max(maxpix, w * h);
+        maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
     }
-    *launched = (plain ? 1 : 0) + (maxtiles ? 1 : 0);
+    plain |= tiles == 0;   // a launch without images still publishes
+    *launched = (plain ? 1 : 0) + (tiles ? 1 : 0);
     const unsigned views = vt.n ? vt.n : 1;
-    if (maxtiles) {   // at most 512 x 512 tiles
-        const cudaError_t e = launch_early(k_resolve_dilated, dim3((unsigned)maxtiles, views), 256, st, c, vt,
-                                           view_base, s, publish && !plain);
+    if (tiles) {
+        const cudaError_t e = launch_early(k_resolve_dilated, dim3(tiles), 256, st, c, vt, grid, view_base, s,
+                                           publish && !plain);
         if (e != cudaSuccess || !plain) return e;
     }
     // one or four pixels per thread
