@@ -1527,11 +1527,13 @@ __device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counte
     return __shfl_sync(FULL, i, 0);
 }
 
-// The colour pass walks the list in another order: kFan places far apart in the
-// list in turn. Neighbouring entries add to the same pixels' sums, and the warps
-// that run at one time then wait for one another's reductions (200M-point
+// The colour pass with two-word sums walks the list in another order: kFan places far
+// apart in the list in turn. Neighbouring entries add to the same pixels' sums, and the
+// warps that run at one time then wait for one another's reductions (200M-point
 // overview: 724 us in list order, 704 / 685 / 643 / 656 us with 8 / 64 / 1024 / 8192 places;
-// the depth pass gains nothing from it).
+// frames of 100M points at 1080p: one view 615 -> 584 us, two 776 -> 759, eight 2,929 ->
+// 2,858). The depth pass gains nothing from it, and packed sums, which wait for each
+// addition's old value, lose (four views 2,981 -> 3,144 us): they keep the list's order.
 constexpr uint32_t kFan = 1024u;
 __device__ __forceinline__ uint32_t fan_out(uint32_t i, uint32_t n) {
     const uint32_t rounds = n / kFan;   // the places' lengths; the rest stays in order
@@ -2134,7 +2136,8 @@ __global__ void __launch_bounds__(256, 4) k_shade(CloudView c, ViewTable vt, Scr
     n_entries += n_front;
     for (uint32_t i = first_entry(n_entries); i < n_entries;
          i = next_entry(s, FALLBACK ? C_GRAB_FALLBACK : C_GRAB_SHADE, n_entries, lane)) {
-        const DrawEntry e = s.entries[i < n_front ? fan_out(i, n_front) : s.capacity - 1u - (i - n_front)];
+        const uint32_t front = LAYOUTS == 1 ? fan_out(i, n_front) : i;
+        const DrawEntry e = s.entries[i < n_front ? front : s.capacity - 1u - (i - n_front)];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
             continue;
