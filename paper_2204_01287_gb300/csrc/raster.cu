@@ -297,6 +297,89 @@ __device__ __forceinline__ BatchTest test_batch(const pc_batch& b, const ViewPar
     return r;
 }
 
+// The same tests by one thread, each with the operations of test_batch and only where
+// its result is asked for. A team shortens the chain of a batch's tests; where there are
+// batches enough to fill the chip, one thread each takes a third of the instructions.
+__device__ __forceinline__ void batch_box(const pc_batch& b, float (&lo)[3], float (&hi)[3]) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = b.min[a];
+        hi[a] = __fadd_rn(b.min[a], b.size[a]);
+    }
+}
+
+__device__ __forceinline__ bool culled_alone(const pc_batch& b, const ViewParams& v) {
+    const float g = 6.0f * 0x1.0p-24f, e1 = 1.0f + 0x1.0p-10f, band = 0x1.0p-16f;
+    float lo[3], hi[3];
+    batch_box(b, lo, hi);
+    const float* m = v.m;
+    const float Wr[4] = {m[3], m[7], m[11], m[15]};
+    const float bw = row_mag32(Wr, lo, hi);
+    bool bad = !(bw <= 0x1.0p100f) || !(bw >= 0x1.0p-90f), out = false, open = false;
+    auto plane = [&](const float (&r)[4], float mag) {
+        const float t = __fadd_rn(row_max32(r, lo, hi), __fmul_rn(g, mag)), lim = __fmul_rn(band, mag);
+        out |= t < -lim;
+        open |= !(t < -lim) && !(t > lim);
+    };
+    plane(Wr, bw);
+#pragma unroll
+    for (int axis = 0; axis < 2; ++axis) {
+        const float R[4] = {m[axis], m[4 + axis], m[8 + axis], m[12 + axis]};
+        const float mag = __fadd_rn(row_mag32(R, lo, hi), __fmul_rn(e1, bw));
+        bad |= !(mag <= 0x1.0p100f) || !(mag >= 0x1.0p-90f);
+        float low[4], high[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            low[a] = __fadd_rn(R[a], __fmul_rn(e1, Wr[a]));
+            high[a] = __fadd_rn(-R[a], __fmul_rn(e1, Wr[a]));
+        }
+        plane(low, mag);
+        plane(high, mag);
+    }
+    return bad || (open && !out) ? cull_batch_exact(b, v) : out;
+}
+
+__device__ __forceinline__ void corners_alone(const pc_batch& b, const ViewParams& v, BatchTest& t) {
+    float lo[3], hi[3];
+    batch_box(b, lo, hi);
+    t.front = true;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const float x = (c & 1) ? hi[0] : lo[0], y = (c & 2) ? hi[1] : lo[1], z = (c & 4) ? hi[2] : lo[2];
+        const float cw = clip_row(v.m, 3, x, y, z);
+        t.front = t.front && cw > 0.0f;
+        const float f0 = to_pixel(clip_row(v.m, 0, x, y, z), cw, (float)v.width);
+        const float f1 = to_pixel(clip_row(v.m, 1, x, y, z), cw, (float)v.height);
+        // a NaN of corner 0 stays, a NaN of a later one is passed over
+        if (c == 0 || f0 < t.fmin0) t.fmin0 = f0;
+        if (c == 0 || f0 > t.fmax0) t.fmax0 = f0;
+        if (c == 0 || f1 < t.fmin1) t.fmin1 = f1;
+        if (c == 0 || f1 > t.fmax1) t.fmax1 = f1;
+    }
+}
+
+__device__ __forceinline__ bool inside_alone(const pc_batch& b, const ViewParams& v) {
+    if ((v.flags & PC_VIEW_NO_EARLY_DEPTH) || !(b.size[0] <= 0x1.0p100f) || !(b.size[1] <= 0x1.0p100f) ||
+        !(b.size[2] <= 0x1.0p100f))
+        return false;
+    const float g = 32.0f * 0x1.0p-24f, tiny = 0x1.0p-120f, lim = 1.0f - 0x1.0p-12f;
+    float lo[3], hi[3];
+    batch_box(b, lo, hi);
+    const float* m = v.m;
+    const float Wr[4] = {m[3], m[7], m[11], m[15]};
+    const float mw = __fadd_rn(__fmul_rn(g, row_mag32(Wr, lo, hi)), tiny);
+    const float wl = __fsub_rn(row_min32(Wr, lo, hi), mw), wh = __fadd_rn(row_max32(Wr, lo, hi), mw);
+    bool ok = wl >= 0x1.0p-99f && wh <= 0x1.0p99f;
+#pragma unroll
+    for (int axis = 0; axis < 2; ++axis) {
+        const float R[4] = {m[axis], m[4 + axis], m[8 + axis], m[12 + axis]};
+        const float mr = __fadd_rn(__fmul_rn(g, row_mag32(R, lo, hi)), tiny);
+        const float cl = __fsub_rn(row_min32(R, lo, hi), mr), ch = __fadd_rn(row_max32(R, lo, hi), mr);
+        ok = ok && __fdiv_rn(cl, cl >= 0.0f ? wh : wl) >= -lim && __fdiv_rn(ch, ch >= 0.0f ? wl : wh) <= lim;
+    }
+    return ok;
+}
+
 // Sec. 3.3: smallest k whose cells are below the threshold, from the extent
 // of the 8 projected box corners; 3 when a corner is not in front of the eye.
 __device__ __forceinline__ int select_k(const BatchTest& t, uint32_t flags, float T) {
@@ -414,7 +497,7 @@ __device__ void append_batches(CullShared& sh, uint32_t first, uint32_t n, const
         }
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x >> 3; i < n; i += kCullTeams) {
+    for (uint32_t i = threadIdx.x >> 3; i < n; i += blockDim.x >> 3) {
         const LodSel sel = sh.sel[i];
         const bool general = vt.n == 1 && !(sel.fast & 1u);
         const uint32_t count = sh.count[i], nseg = sh.nseg[i];
@@ -467,9 +550,8 @@ __device__ __forceinline__ void init_cull(CullShared& sh, uint32_t nviews) {
 // when its ancestors pass too: k_lod_append).
 // Bound by latency: the batch's load, the tests' chain and one atomic. One thread
 // per batch, with the views in turn, and a clear pass before it took 19 us for a
-// 1M-point cloud at 512x512 (65 us with 16 views, 43 us for 2B points at 1080p);
-// this pass takes 11 us (25 and 39 us). Four blocks per SM (64 registers): with
-// the 89 registers it would take, the 2B frame's 195,313 batches need 53 us.
+// 1M-point cloud at 512x512 and 65 us with 16 views; this pass takes 11 and 25 us.
+// Four blocks per SM (64 registers). Clouds of many batches take k_begin_many.
 __global__ void __launch_bounds__(kCullThreads, 4) k_begin(CloudView c, ViewTable vt, Scratch s,
                                                       uint32_t cull_blocks, uint32_t per_block,
                                                       uint32_t clear_parts) {
@@ -514,6 +596,75 @@ __global__ void __launch_bounds__(kCullThreads, 4) k_begin(CloudView c, ViewTabl
         for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s.lod_sel[first + i] = sh.sel[i];
         return;
     }
+    append_batches(sh, first, n, vt, s);
+}
+
+// The first pass for many batches (launch_begin chooses): one thread per batch, the
+// views in turn, each test only where its result is needed. Bound by instruction
+// issue: about 100 binary32 operations a test that culls, 400 one that does not.
+__global__ void __launch_bounds__(kCullBatches, 8) k_begin_many(CloudView c, ViewTable vt, Scratch s,
+                                                             uint32_t cull_blocks, uint32_t clear_parts) {
+    start_next();
+    wait_for_previous();
+    if (blockIdx.x >= cull_blocks) {
+        const uint32_t j = blockIdx.x - cull_blocks;
+        clear_view(vt.v[j / clear_parts], j % clear_parts, clear_parts);
+        return;
+    }
+    __shared__ CullShared sh;
+    init_cull(sh, vt.n);
+    __syncthreads();
+    const uint32_t first = blockIdx.x * kCullBatches, n = min(kCullBatches, c.n_batches - first);
+    const uint32_t i = threadIdx.x;
+    pc_batch bt{};
+    uint32_t count = 0;
+    if (i < n) {
+        bt = c.batches[first + i];
+        count = bt.count;
+        if ((uint64_t)bt.first + bt.count > c.n_points) {
+            raise_error(s, E_BATCH_RANGE, first + i);
+            count = 0;
+        }
+    }
+    const bool test = i < n && (count || c.is_lod);
+    LodSel e{};
+    for (uint32_t v = 0; v < vt.n; ++v) {
+        const ViewParams& vp = vt.v[v];
+        int k = 0;
+        if (test) {
+            BatchTest t{};
+            t.culled = (c.is_lod || (vp.flags & PC_VIEW_CULL)) && culled_alone(bt, vp);
+            if (!t.culled) {
+                if (!(vp.flags & PC_VIEW_K_MASK) || c.is_lod) corners_alone(bt, vp, t);
+                if (!c.is_lod || lod_passes(t, vp, first + i == 0)) {
+                    k = select_k(t, vp.flags, vt.threshold_px);
+                    e.mask |= 1u << v;
+                    e.kcodes |= (unsigned long long)k << (2u * v);
+                    if (k <= 2 && inside_alone(bt, vp)) e.fast |= 1u << v;
+                }
+            }
+        }
+        if (c.is_lod || !__any_sync(FULL, k != 0)) continue;
+        // the statistics, summed over the warp first
+#pragma unroll
+        for (int kk = 1; kk <= 3; ++kk) {
+            const uint32_t nb = __popc(__ballot_sync(FULL, k == kk));
+            if (!nb) continue;
+            const uint32_t own = k == kk ? count : 0u;
+            const uint32_t lo = __reduce_add_sync(FULL, own & 0xFFFFu), hi = __reduce_add_sync(FULL, own >> 16);
+            if ((i & 31u) != 0u) continue;
+            atomicAdd(&sh.batches[v][kk - 1], nb);
+            atomicAdd(&sh.lo[v][kk - 1], lo);
+            atomicAdd(&sh.hi[v][kk - 1], hi);
+        }
+    }
+    if (c.is_lod) {
+        if (i < n) s.lod_sel[first + i] = e;
+        return;
+    }
+    sh.sel[i] = e;
+    sh.count[i] = count;
+    __syncthreads();
     append_batches(sh, first, n, vt, s);
 }
 
@@ -2491,17 +2642,32 @@ static uint32_t cull_batches_per_block(uint32_t n_batches, uint32_t nviews) {
     return std::min(kCullBatches, std::max(round, spread));
 }
 
+// Batches from which the first pass takes one thread per batch. Clear and cull of views
+// of 64x48, with a team of lanes per batch and view / with one thread per batch (us):
+//   batches     1 view       4 views      32 views     (everything in view)
+//    1,000   10.8 / 12.8   10.8 / 17.1   32.9 / 61.9
+//    8,000   10.6 / 12.7   16.1 / 17.1   45.3 / 61.9
+//   16,000   11.7 / 12.6   20.8 / 17.3   79.1 / 67.9
+//   32,000   16.7 / 13.5   28.9 / 18.8    148 / 74.0
+//  340,000   54.1 / 34.1    158 / 54.7  1,127 / 294
+// A few batches are a matter of latency, which the team shortens; many are one of
+// instructions. The two meet between 8,000 and 32,000 batches for any number of views.
+constexpr uint32_t kManyBatches = 16384;
+
 cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
     uint64_t maxpix = 0;
     for (uint32_t v = 0; v < vt.n; ++v)
         maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
-    // the views share eight clearing blocks per SM
-    const uint64_t most = std::max<uint64_t>(1, (uint64_t)num_sms() * 8 / std::max(1u, vt.n));
-    const uint64_t parts = std::min(most, std::max<uint64_t>(1, (maxpix / 2 + kCullThreads - 1) / kCullThreads));
-    const uint32_t per = cull_batches_per_block(c.n_batches, vt.n);
+    // the views share eight clearing blocks of 256 threads per SM
+    const bool many = c.n_batches >= kManyBatches;
+    const uint32_t threads = many ? kCullBatches : kCullThreads;
+    const uint64_t most = std::max<uint64_t>(1, (uint64_t)num_sms() * 8 * kCullThreads / threads / std::max(1u, vt.n));
+    const uint64_t parts = std::min(most, std::max<uint64_t>(1, (maxpix / 2 + threads - 1) / threads));
+    const uint32_t per = many ? kCullBatches : cull_batches_per_block(c.n_batches, vt.n);
     const uint32_t cull = (c.n_batches + per - 1) / per;
-    return launch_early(k_begin, dim3(cull + (uint32_t)parts * vt.n), kCullThreads, st, c, vt, s, cull, per,
-                        (uint32_t)parts);
+    const dim3 grid(cull + (uint32_t)parts * vt.n);
+    if (many) return launch_early(k_begin_many, grid, threads, st, c, vt, s, cull, (uint32_t)parts);
+    return launch_early(k_begin, grid, threads, st, c, vt, s, cull, per, (uint32_t)parts);
 }
 
 cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
