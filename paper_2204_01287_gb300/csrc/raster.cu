@@ -1671,11 +1671,27 @@ __device__ __forceinline__ uint32_t first_entry(uint32_t n) {
     const uint32_t share = min(per_block, max(4u, (n + gridDim.x - 1u) / gridDim.x));
     return __shfl_sync(FULL, w < share ? blockIdx.x * share + w : n, 0);
 }
+// given: entries taken without the counter.
+__device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counter, uint32_t n,
+                                               uint32_t lane, uint32_t given) {
+    uint32_t i = n;
+    if (lane == 0 && n > given) i = given + atomicAdd(&s.counters[counter], 1u);
+    return __shfl_sync(FULL, i, 0);
+}
 __device__ __forceinline__ uint32_t next_entry(const Scratch& s, uint32_t counter, uint32_t n,
                                                uint32_t lane) {
-    uint32_t i = n;
-    if (lane == 0 && n > grid_warps()) i = grid_warps() + atomicAdd(&s.counters[counter], 1u);
-    return __shfl_sync(FULL, i, 0);
+    return next_entry(s, counter, n, lane, grid_warps());
+}
+
+// One-view launches of a long list into a small image take every entry from the counter:
+// when all warps start at once, their first points all find empty pixels, and the
+// atomics on the few there are queue up; the counter lets the warps in one after the
+// other. Frames with static first entries / this way (us): 5M points seen whole at 16x9
+// 136 / 103, 200M points along a fly-through at 16x9 105 / 75, at 64x36 128 / 105, at
+// 160x90 73 / 65. Lists of one round lose by it (5M points at 160x90 17.5 / 21.7), and so do
+// larger images (the raster pass at 320x180 28 / 33).
+__device__ __forceinline__ bool few_pixels(uint32_t npix, uint32_t n) {
+    return npix <= 16384u && n > grid_warps();
 }
 
 // The colour pass with two-word sums walks the list in another order: kFan places far
@@ -1766,7 +1782,10 @@ __global__ void __launch_bounds__(kRasterThreads, 5) k_raster_fast(CloudView c,
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t n_entries = take_list(s);
     uint32_t n_atom = 0;
-    for (uint32_t i = first_entry(n_entries); i < n_entries; i = next_entry(s, C_GRAB, n_entries, lane)) {
+    const bool few = few_pixels(fv.npix, n_entries);
+    const uint32_t given = few ? 0u : grid_warps();
+    for (uint32_t i = few ? next_entry(s, C_GRAB, n_entries, lane, 0u) : first_entry(n_entries); i < n_entries;
+         i = next_entry(s, C_GRAB, n_entries, lane, given)) {
         const DrawEntry e = s.entries[i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
@@ -1800,8 +1819,10 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView 
     }
     const ViewConst vc = make_view_const(vt.v[0]);
     uint32_t n_atom = 0;
-    for (uint32_t i = first_entry(n_entries); i < n_entries;
-         i = next_entry(s, C_GRAB_GENERAL, n_entries, lane)) {
+    const bool few = few_pixels(vc.width * vc.height, n_entries);
+    const uint32_t given = few ? 0u : grid_warps();
+    for (uint32_t i = few ? next_entry(s, C_GRAB_GENERAL, n_entries, lane, 0u) : first_entry(n_entries);
+         i < n_entries; i = next_entry(s, C_GRAB_GENERAL, n_entries, lane, given)) {
         const DrawEntry e = s.entries[s.capacity - 1u - i];
         if (e.batch >= c.n_batches) {
             if (lane == 0) raise_error(s, E_BATCH_RANGE, e.batch);
