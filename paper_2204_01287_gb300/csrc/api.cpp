@@ -68,21 +68,15 @@ CloudView Cloud::view() const {
 
 Slot::~Slot() {
     for (auto& kv : graphs) cudaGraphExecDestroy(kv.second);
+    if (branch.side) cudaStreamDestroy(branch.side);
+    if (branch.fork) cudaEventDestroy(branch.fork);
+    if (branch.join) cudaEventDestroy(branch.join);
     cudaFree(scratch.entries);
     cudaFree(scratch.counters);
     cudaFree(scratch.lod_sel);
     cudaFree(hqs_accum);
     cudaFree(host_vis);
     cudaFree(host_rgba);
-}
-
-// True while the stream is being captured: work on it is then recorded and has not
-// run (also taken for true when the stream cannot be asked).
-static bool capturing(cudaStream_t st) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
-    cudaGetLastError();
-    return true;
 }
 
 // Zero, in stream order, of what a frame's last pass leaves at zero (the sums, and the
@@ -100,6 +94,22 @@ static cudaError_t clear_scratch(const Slot& s, bool all) {
         e = cudaMemsetAsync(s.scratch.counters + C_ERRINFO + 1, 0,
                             sizeof(uint32_t) * (C_LIST - C_ERRINFO - 1), s.stream);
     return e;
+}
+
+// What captured frames need for two branches, made by the first one; nullptr when it
+// cannot be had (the frame's kernels then follow one another).
+const Branch* Slot::second_branch() {
+    if (branch.join) return &branch;
+    // allowed in every capture mode: nothing here touches a captured stream
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return nullptr;
+    cudaError_t e = cudaSuccess;
+    if (!branch.side) e = cudaStreamCreateWithFlags(&branch.side, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !branch.fork) e = cudaEventCreateWithFlags(&branch.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&branch.join, cudaEventDisableTiming);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess ? &branch : nullptr;
 }
 
 pc_status Ctx::ensure_capacity(Slot& s, uint64_t entries, uint64_t nodes) {
@@ -233,7 +243,8 @@ uint32_t Ctx::views_per_launch(const Cloud& cl) const {
 // resolve. *kernels: how many.
 pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                             const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
-                            uint32_t maxv, bool timing, const FrameOpts& fo, uint32_t* kernels) {
+                            uint32_t maxv, bool timing, bool captured, const FrameOpts& fo,
+                            uint32_t* kernels) {
     CloudView cv = cl.view();
     if (fo.first || fo.count < cl.n_batches) {
         // a shard: the kernels see only the batches of the range (their point
@@ -300,8 +311,10 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         }
         if (fe) cudaEventRecord(fe->ev[2], st);
         int raster_kernels = 0;
-        slot->scratch.frame = next_frame(slot->scratch.frame);
-        e = launch_raster(cv, vt, slot->scratch, shape, st, &raster_kernels);
+        Scratch s = slot->scratch;
+        s.frame = 0;
+        if (!captured) s.frame = slot->scratch.frame = next_frame(slot->scratch.frame);
+        e = launch_raster(cv, vt, s, shape, captured ? slot->second_branch() : nullptr, st, &raster_kernels);
         if (e != cudaSuccess) return cuda_fail(e, "raster launch");
         if (fe) cudaEventRecord(fe->ev[3], st);
         if (shade) {
@@ -390,7 +403,7 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
     uint32_t kernels = 0;
-    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, fo, &kernels);
+    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, graph || capturing(st), fo, &kernels);
     launches += kernels;
     if (rc != PC_OK && !graph) {
         // The last pass, which leaves the scratch at zero, is missing: clear it behind

@@ -105,7 +105,7 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     s.stats = L->stats;
     s.lod_sel = nullptr;
     static std::atomic<uint64_t> calls{0};   // numbers 1, 2, ... of the process's calls
-    s.frame = (uint32_t)(calls.fetch_add(1u) % 0xFFFFFFFFu) + 1u;
+    s.frame = capturing(st) ? 0u : (uint32_t)(calls.fetch_add(1u) % 0xFFFFFFFFu) + 1u;
     // the array keeps the previous call's contents: counters and sums
     // (including the error flag) start from zero every call
     if (cudaMemsetAsync(L->counters, 0, sizeof L->counters + sizeof L->acc, st) != cudaSuccess)
@@ -140,7 +140,7 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     shape.blocks = 0;   // one resident wave
     if (launch_begin(c, vt, s, st) != cudaSuccess) return PC_ECUDA;
     int launched = 0;
-    if (nbatches && launch_raster(c, vt, s, shape, st, &launched) != cudaSuccess)
+    if (nbatches && launch_raster(c, vt, s, shape, nullptr, st, &launched) != cudaSuccess)
         return PC_ECUDA;
     if (launch_resolve(c, vt, 0, s, true, st, &launched) != cudaSuccess) return PC_ECUDA;
     // the device error flag and its value, for the caller to read once the

@@ -71,6 +71,8 @@ struct Slot {
     uint32_t last_nviews = 0;
     uint64_t last_total_batches = 0;
     std::map<uint64_t, cudaGraphExec_t> graphs;   // replayable frames by launch layout
+    Branch branch{};                // of captured frames
+    const Branch* second_branch();
     ~Slot();
 };
 
@@ -123,7 +125,7 @@ struct Ctx {
     void set_tune(Cloud& cl, uint32_t nviews, const Tune& t);
     pc_status launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                            const pc_framebuffer* fbs, cudaStream_t st, Slot* slot, uint32_t maxv,
-                           bool timing, const FrameOpts& fo, uint32_t* kernels);
+                           bool timing, bool captured, const FrameOpts& fo, uint32_t* kernels);
     pc_status render(const Cloud& cl, const pc_view* views, uint32_t nviews,
                      const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
                      const FrameOpts& fo = FrameOpts());

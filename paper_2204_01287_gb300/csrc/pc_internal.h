@@ -156,12 +156,21 @@ struct Scratch {
                                 // progress. acc and the counters before C_LIST (the
                                 // error words apart) are zero between launches;
                                 // k_resolve leaves them so
-    uint32_t frame;       // number of this launch (next_frame)
+    uint32_t frame;       // number of this launch (next_frame); 0 while it is captured
     LodSel* lod_sel;      // LOD: per node
 };
 
 // The number of the launch after `last`: any but 0, which a cleared scratch holds.
 inline uint32_t next_frame(uint32_t last) { return last == ~0u ? 1u : last + 1u; }
+
+// True while the stream is being captured: work on it is then recorded and has not
+// run (also taken for true when the stream cannot be asked).
+inline bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess) return cs != cudaStreamCaptureStatusNone;
+    cudaGetLastError();
+    return true;
+}
 
 // Launch-shape knobs for the raster kernel.
 struct RasterShape {
@@ -175,8 +184,16 @@ struct RasterShape {
 // cloud, writes the draw list; for an LOD cloud launch_lod_append writes it.
 cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
 cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
-// *launched: kernels launched.
-cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s, RasterShape shape, cudaStream_t st, int* launched);
+// A stream and two events with which a captured frame becomes two branches for the two
+// one-view kernels (a graph has no early starts: one after the other they would wait
+// for one another's last blocks).
+struct Branch {
+    cudaStream_t side;
+    cudaEvent_t fork, join;
+};
+// *launched: kernels launched. branch: for captured launches, or nullptr.
+cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s, RasterShape shape,
+                          const Branch* branch, cudaStream_t st, int* launched);
 // High-quality shading colour pass (Sec. 3.6) over the draw list of the
 // launch, for the views with a sum buffer, and the fallback pass of packed
 // views; after launch_raster. *launched: kernels launched.

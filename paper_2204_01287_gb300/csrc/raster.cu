@@ -1721,8 +1721,9 @@ __device__ __forceinline__ void entry_counts(const Scratch& s, uint32_t& front, 
 // sees all that was visible to that thread: the list, the counters and the cleared
 // keys. An older number (the store has not arrived, or another kernel was queued
 // between the two) takes the wait, after which the same holds. A frame's number is
-// never 0 and differs from those before it in the same scratch; a replayed graph
-// repeats its number, but its kernels run one after the other.
+// never 0 and differs from those before it in the same scratch. Captured launches, whose
+// number would come again with every replay, have none: there both kernels start when
+// the first pass has ended, and read the counters.
 __device__ __forceinline__ void give_list(const Scratch& s, uint32_t front) {
     asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(s.counters + C_LIST),
                  "l"((unsigned long long)s.frame << 32 | front)
@@ -1737,7 +1738,7 @@ __device__ __forceinline__ uint32_t take_list(const Scratch& s) {
     }
     __syncthreads();
     uint32_t front = (uint32_t)given;
-    if ((uint32_t)(given >> 32) != s.frame) {
+    if (s.frame == 0u || (uint32_t)(given >> 32) != s.frame) {
         uint32_t back;
         wait_for_previous();
         entry_counts(s, front, back);
@@ -1806,7 +1807,7 @@ __global__ void __launch_bounds__(kRasterThreads, 4) k_raster_general(CloudView 
     wait_for_previous();
     const uint32_t lane = threadIdx.x & 31;
     uint32_t n_front, n_entries;
-    if (blockIdx.x == 0) {
+    if (blockIdx.x == 0 && s.frame != 0u) {
         // the fast kernel starts when every block has come past start_next, by
         // which time the list is on its way
         entry_counts(s, n_front, n_entries);
@@ -2643,13 +2644,8 @@ static cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, unsigned t
     // since graphs are what programs replay on several streams at once (16 views of
     // 1M points on three streams: 80 us a frame with early starts, 66 us without; one
     // view of 10M points on one stream: 28 and 30 us).
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) {
-        cudaGetLastError();   // plain edges are always right; the launch reports what is wrong
-        capture = cudaStreamCaptureStatusActive;
-    }
     cfg.attrs = &early;
-    cfg.numAttrs = capture == cudaStreamCaptureStatusNone ? 1 : 0;
+    cfg.numAttrs = capturing(st) ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
@@ -2723,8 +2719,8 @@ static PairView make_pair_view(const ViewParams& v) {
     return pv;
 }
 
-cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
-                          RasterShape shape, cudaStream_t st, int* launched) {
+cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s, RasterShape shape,
+                          const Branch* branch, cudaStream_t st, int* launched) {
     int threads = shape.threads_per_block > 0 ? shape.threads_per_block : kRasterThreads;
     threads = threads > kRasterThreads ? kRasterThreads : (threads < 32 ? 32 : threads & ~31);
     const int blocks = shape.blocks > 0 ? shape.blocks : num_sms() * raster_occupancy(threads, vt.n);
@@ -2732,9 +2728,22 @@ cudaError_t launch_raster(const CloudView& c, const ViewTable& vt, Scratch s,
     if (vt.n > 2) return launch_early(k_rasterN, dim3(blocks), threads, st, c, vt, s);
     if (vt.n == 2) return launch_early(k_raster2, dim3(blocks), threads, st, c, vt, make_pair_view(vt.v[0]),
                                          make_pair_view(vt.v[1]), s);
-    cudaError_t e = launch_early(k_raster_general, dim3(num_sms() * 4), kRasterThreads, st, c, vt, s);
-    if (e != cudaSuccess) return e;
-    return launch_early(k_raster_fast, dim3(blocks), threads, st, c, make_pair_view(vt.v[0]), s);
+    cudaStream_t fast = st;
+    cudaError_t e = cudaSuccess;
+    if (branch) {
+        e = cudaEventRecord(branch->fork, st);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(branch->side, branch->fork, 0);
+        if (e != cudaSuccess) return e;
+        fast = branch->side;
+    }
+    e = launch_early(k_raster_general, dim3(num_sms() * 4), kRasterThreads, st, c, vt, s);
+    if (e == cudaSuccess) e = launch_early(k_raster_fast, dim3(blocks), threads, fast, c, make_pair_view(vt.v[0]), s);
+    if (branch) {   // the branches meet again even when a launch failed: the capture is the caller's
+        cudaError_t j = cudaEventRecord(branch->join, branch->side);
+        if (j == cudaSuccess) j = cudaStreamWaitEvent(st, branch->join, 0);
+        if (e == cudaSuccess) e = j;
+    }
+    return e;
 }
 
 template <int LAYOUTS>

@@ -27,7 +27,8 @@ struct CUgraphExec_st { Ops ops; };
 
 static Ops* g_recording = nullptr;        // the captured stream's work
 static std::map<std::string, int> g_fail; // call -> calls until one fails (1: the next)
-static int g_dirty = 0, g_frames = 0, g_instantiated = 0, g_encoded = 0;
+static int g_dirty = 0, g_frames = 0, g_instantiated = 0, g_encoded = 0, g_branches = 0, g_misnumbered = 0;
+static uint32_t g_last_frame = 0;
 static size_t g_room = ~(size_t)0, g_used = 0;   // bytes the "device" has, and lent
 static std::map<void*, size_t> g_blocks;
 
@@ -77,12 +78,21 @@ cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t) { return "stand-in error"; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = nullptr; return cudaSuccess; }
-cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = nullptr; return cudaSuccess; }
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
+    *e = reinterpret_cast<cudaEvent_t>(0x60);
+    return cudaSuccess;
+}
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* t, cudaEvent_t, cudaEvent_t) { *t = 0.0f; return cudaSuccess; }
-cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = nullptr; return cudaSuccess; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
+    *s = nullptr;
+    if (fails("stream")) return cudaErrorMemoryAllocation;
+    *s = reinterpret_cast<cudaStream_t>(0x50);
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode*) { return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
@@ -143,7 +153,12 @@ cudaError_t launch_lod_append(const CloudView&, const ViewTable&, Scratch, cudaS
     run([] {});
     return cudaSuccess;
 }
-cudaError_t launch_raster(const CloudView&, const ViewTable& vt, Scratch, RasterShape, cudaStream_t, int* launched) {
+cudaError_t launch_raster(const CloudView&, const ViewTable& vt, Scratch s, RasterShape, const Branch* branch,
+                          cudaStream_t, int* launched) {
+    // a captured launch has no number (every replay would repeat it), others one of their own
+    if ((g_recording != nullptr) != (s.frame == 0) || (s.frame && s.frame <= g_last_frame)) ++g_misnumbered;
+    if (s.frame) g_last_frame = s.frame;
+    if (branch) ++g_branches;
     if (fails("raster")) return cudaErrorLaunchFailure;
     *launched = vt.n == 1 ? 2 : 1;
     for (int i = 0; i < *launched; ++i) run([] {});
@@ -375,6 +390,25 @@ static void graphs_of_alternating_layouts() {
     CHECK(g_instantiated == made && g_dirty == 0);
 }
 
+// Captured frames, a caller's and the library's own, have no frame number and run the
+// two one-view kernels as two branches, or as one where a branch cannot be had.
+static void captured_frames_branch() {
+    {
+        World w;
+        CHECK(w.frame() == PC_OK && g_branches == 0);
+        g_fail["stream"] = 1;
+        cudaGraphExecDestroy(captured_frame(w));
+        CHECK(g_branches == 0);
+        cudaGraphExecDestroy(captured_frame(w));
+        CHECK(w.frame() == PC_OK && w.frame() == PC_OK);
+        CHECK(g_branches == 1);
+    }
+    g_last_frame = 0;
+    World w(PC_CFG_GRAPHS);
+    for (int i = 0; i < 3; ++i) CHECK(w.frame() == PC_OK && g_branches == 2 + i);
+    CHECK(g_misnumbered == 0 && g_instantiated == 3 && g_dirty == 0);
+}
+
 static const std::map<std::string, void (*)()>& scenarios() {
     static const std::map<std::string, void (*)()> all = {
         {"failed_frame", failed_frame},
@@ -386,6 +420,7 @@ static const std::map<std::string, void (*)()>& scenarios() {
         {"first_frame_captured", first_frame_captured},
         {"upload_without_room", upload_without_room},
         {"graphs_of_alternating_layouts", graphs_of_alternating_layouts},
+        {"captured_frames_branch", captured_frames_branch},
     };
     return all;
 }
