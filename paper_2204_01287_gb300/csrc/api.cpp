@@ -656,7 +656,7 @@ pc_status upload_encoded_internal(Ctx& c, const pc_batch* batches, uint64_t nbat
 }
 
 // Encodes raw points on the host into a new cloud's device buffers.
-static pc_status encode_on_host(Ctx& c, const float* xyz, const uint32_t* rgba, Cloud& cl) {
+static pc_status encode_on_host(Ctx& c, const float* xyz, const uint32_t* rgba, uint32_t threads, Cloud& cl) {
     std::vector<pc_batch> batches;
     std::vector<uint32_t> words[4];   // three of coordinates, the colours
     try {
@@ -668,7 +668,7 @@ static pc_status encode_on_host(Ctx& c, const float* xyz, const uint32_t* rgba, 
     }
     const uint32_t eflags = (c.cfg.flags & PC_CFG_KEEP_ORDER) ? PC_ENCODE_KEEP_ORDER : 0u;
     const pc_status rc =
-        pc_encode(xyz, rgba, cl.n_points, c.cfg.batch_size, c.cfg.encoder_threads, eflags, batches.data(),
+        pc_encode(xyz, rgba, cl.n_points, c.cfg.batch_size, threads, eflags, batches.data(),
                   words[0].data(), words[1].data(), words[2].data(), words[3].data(), nullptr);
     if (rc != PC_OK) {
         c.fail_msg("encoder failed: %s", pc_strerror(rc));
@@ -684,7 +684,10 @@ static pc_status encode_on_host(Ctx& c, const float* xyz, const uint32_t* rgba, 
 // the host with the same bits.
 // The host encoder took 32 ms for 4M points on 16 cores, half of it in page faults
 // of its arrays; the device takes 1.6 ms: the copy of 64 MB 0.4, the kernels 0.8, the
-// allocations the rest.
+// allocations the rest. A few points kept in their order are encoded by one host thread
+// (1 / 1,000 / 2,000 points: 194 / 222 / 248 us against 216 / 231 / 237 on the device); with
+// the sort the device is faster from the first point on (457 against 396 us).
+constexpr uint64_t kHostPoints = 1000;
 static pc_status upload_points(Ctx& c, const float* xyz, const uint32_t* rgba, uint64_t n,
                                std::shared_ptr<Cloud>& out) {
     const uint32_t bs = c.cfg.batch_size;
@@ -692,8 +695,9 @@ static pc_status upload_points(Ctx& c, const float* xyz, const uint32_t* rgba, u
     const uint64_t nb = (n + bs - 1) / bs, last = n - (nb - 1) * bs;
     const uint64_t entries = (nb - 1) * ((bs + kMinSegmentPoints - 1) / kMinSegmentPoints) +
                              (last + kMinSegmentPoints - 1) / kMinSegmentPoints;
+    const bool few = keep && n <= kHostPoints;
     void* scratch = nullptr;
-    if (cudaMalloc(&scratch, encode_device_scratch(n, rgba != nullptr, keep)) != cudaSuccess) {
+    if (!few && cudaMalloc(&scratch, encode_device_scratch(n, rgba != nullptr, keep)) != cudaSuccess) {
         cudaGetLastError();
         scratch = nullptr;
     }
@@ -707,7 +711,7 @@ static pc_status upload_points(Ctx& c, const float* xyz, const uint32_t* rgba, u
     }
     if (rc != PC_OK) rc = allocation_failed(c, rc, e, n);
     if (rc == PC_OK && !scratch) {
-        rc = encode_on_host(c, xyz, rgba, *cl);
+        rc = encode_on_host(c, xyz, rgba, few ? 1u : c.cfg.encoder_threads, *cl);
     } else if (rc == PC_OK) {
         bool finite = false;
         e = encode_device(xyz, rgba, n, bs, keep, scratch, cl->batches, cl->w1, cl->w2, cl->w3, cl->color,

@@ -375,6 +375,19 @@ static void upload_without_room() {
     CHECK(pc_cloud_get_info(w.ctx, c, &info) == PC_OK && info.n_points == 0 && info.n_batches == 0);
 }
 
+// A few points kept in their order are the host's, more and sorted ones the device's.
+static void few_points_are_encoded_on_the_host() {
+    for (uint32_t flags : {0u, (uint32_t)PC_CFG_KEEP_ORDER})
+        for (uint64_t n : {1, 1000, 1001}) {
+            g_encoded = 0;
+            World w(flags, n);
+            CHECK(g_encoded == !(flags && n <= 1000));
+            pc_cloud c = 0;
+            w.xyz[0] = NAN;
+            CHECK(pc_upload_cloud(w.ctx, w.xyz.data(), nullptr, n, &c) == PC_EINVAL && c == 0);
+        }
+}
+
 // PC_CFG_GRAPHS: a program that alternates between launch layouts of one view count
 // instantiates one graph for each and then only updates.
 static void graphs_of_alternating_layouts() {
@@ -419,6 +432,7 @@ static const std::map<std::string, void (*)()>& scenarios() {
         {"first_clearing_fails", first_clearing_fails},
         {"first_frame_captured", first_frame_captured},
         {"upload_without_room", upload_without_room},
+        {"few_points_are_encoded_on_the_host", few_points_are_encoded_on_the_host},
         {"graphs_of_alternating_layouts", graphs_of_alternating_layouts},
         {"captured_frames_branch", captured_frames_branch},
     };
