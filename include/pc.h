@@ -383,8 +383,8 @@ typedef struct {
     uint32_t frames;            /* pc_render calls recorded */
     uint32_t launches;          /* kernels launched by those calls */
     double   ms_clear, ms_cull, ms_raster, ms_shade, ms_resolve;  /* summed over frames;
-                                   ms_cull: the clear and the culling, one launch (ms_clear,
-                                   the time before it, is the events' own);
+                                   while they are recorded, the clear and the culling,
+                                   one launch otherwise, follow one another;
                                    ms_shade: the colour pass of high-quality shading */
     uint64_t raster_launches;
 } pc_timing;

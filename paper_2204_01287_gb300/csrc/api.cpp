@@ -301,8 +301,13 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
             *kernels += resolve_kernels;
             continue;
         }
-        if (fe) cudaEventRecord(fe->ev[1], st);   // the clear runs beside the culling
-        e = launch_begin(cv, vt, slot->scratch, st);
+        if (fe) {
+            e = launch_begin(cv, vt, slot->scratch, Begin::kClear, st);
+            if (e != cudaSuccess) return cuda_fail(e, "clear launch");
+            cudaEventRecord(fe->ev[1], st);
+            *kernels += 1;
+        }
+        e = launch_begin(cv, vt, slot->scratch, fe ? Begin::kCull : Begin::kBoth, st);
         if (e != cudaSuccess) return cuda_fail(e, "cull launch");
         if (cl.is_lod) {
             e = launch_lod_append(cv, vt, slot->scratch, st);

@@ -138,7 +138,7 @@ extern "C" pc_status pc_render_noalloc(const pc_batch* batches, uint64_t nbatche
     RasterShape shape;
     shape.threads_per_block = 256;
     shape.blocks = 0;   // one resident wave
-    if (launch_begin(c, vt, s, st) != cudaSuccess) return PC_ECUDA;
+    if (launch_begin(c, vt, s, Begin::kBoth, st) != cudaSuccess) return PC_ECUDA;
     int launched = 0;
     if (nbatches && launch_raster(c, vt, s, shape, nullptr, st, &launched) != cudaSuccess)
         return PC_ECUDA;

@@ -181,8 +181,10 @@ struct RasterShape {
 // ---- kernel launchers (raster.cu) ----------------------------------------
 
 // Clears the views' buffers, tests every batch against every view and, for a plain
-// cloud, writes the draw list; for an LOD cloud launch_lod_append writes it.
-cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
+// cloud, writes the draw list; for an LOD cloud launch_lod_append writes it. Frames
+// timed pass by pass take the clear and the culling one after the other.
+enum class Begin { kBoth, kClear, kCull };
+cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, Begin what, cudaStream_t st);
 cudaError_t launch_lod_append(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st);
 // A stream and two events with which a captured frame becomes two branches for the two
 // one-view kernels (a graph has no early starts: one after the other they would wait

@@ -2671,7 +2671,7 @@ static uint32_t cull_batches_per_block(uint32_t n_batches, uint32_t nviews) {
 // instructions. The two meet between 8,000 and 32,000 batches for any number of views.
 constexpr uint32_t kManyBatches = 16384;
 
-cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cudaStream_t st) {
+cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, Begin what, cudaStream_t st) {
     uint64_t maxpix = 0;
     for (uint32_t v = 0; v < vt.n; ++v)
         maxpix = max(maxpix, (uint64_t)vt.v[v].width * vt.v[v].height);
@@ -2681,8 +2681,10 @@ cudaError_t launch_begin(const CloudView& c, const ViewTable& vt, Scratch s, cud
     const uint64_t most = std::max<uint64_t>(1, (uint64_t)num_sms() * 8 * kCullThreads / threads / std::max(1u, vt.n));
     const uint64_t parts = std::min(most, std::max<uint64_t>(1, (maxpix / 2 + threads - 1) / threads));
     const uint32_t per = many ? kCullBatches : cull_batches_per_block(c.n_batches, vt.n);
-    const uint32_t cull = (c.n_batches + per - 1) / per;
-    const dim3 grid(cull + (uint32_t)parts * vt.n);
+    const uint32_t cull = what == Begin::kClear ? 0u : (c.n_batches + per - 1) / per;
+    const uint32_t clear = what == Begin::kCull ? 0u : (uint32_t)parts;
+    const dim3 grid(cull + clear * vt.n);
+    if (grid.x == 0) return cudaSuccess;
     if (many) return launch_early(k_begin_many, grid, threads, st, c, vt, s, cull, (uint32_t)parts);
     return launch_early(k_begin, grid, threads, st, c, vt, s, cull, per, (uint32_t)parts);
 }
