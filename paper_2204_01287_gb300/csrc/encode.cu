@@ -11,9 +11,10 @@
 //                word split, colours
 //
 // Every binary64 operation is an explicit round-to-nearest intrinsic in the
-// host encoder's order. Bound by binary64 division (six a point; GB300 has 2
-// binary64 FMAs per clock and SM) and, for large clouds, by the sort's
-// scattered writes.
+// host encoder's order, or certified to give its result (quantize). For 4M points
+// the kernels take 0.8 ms: the sort 0.5 (each pass reads and writes 12 bytes a point,
+// 41 of its 63 us in the scatter), k_quantize 0.17 (gathers of 12 bytes by index, nine
+// binary64 operations a point; GB300 has 2 binary64 FMAs per clock and SM), k_codes 0.11.
 #include <algorithm>
 #include <cstdint>
 
@@ -29,6 +30,7 @@ constexpr uint32_t kItems = 16;                       // points per thread of a 
 constexpr uint32_t kTilePoints = kThreads * kItems;   // a warp owns 512 consecutive ones
 constexpr uint32_t kDigits = 256, kPasses = 8;
 constexpr uint32_t kChunk = 2048;                     // counts per block of the scan
+constexpr uint32_t kBlocksPerSm = 8;                  // of the kernels that stride over the points
 
 // What k_bounds leaves: the box's minima and maxima as ordered integers, and
 // whether some coordinate is NaN or infinite.
@@ -83,13 +85,16 @@ __global__ void __launch_bounds__(kThreads) k_bounds(const float* xyz, uint32_t 
 }
 
 // floor(scale * (p - lo) / size) in the host encoder's binary64 operations, clamped
-// to [0, scale - 1]; scale is 2^21 or 2^30 and inv about scale / size. t' = (p - lo) inv is
-// within 3 * 2^-53 of the exact quotient, relatively, and so is the definition's
-// rounded one: both lie within 2^-21 of each other below 2^31. Added to 2^32, t' is rounded
-// to 2^-20, and when that leaves its fraction at neither end of [0, 1) the whole part is
-// the definition's. Otherwise, and for every t' that is not in [0, 2^32), the
-// definition decides. Three binary64 operations in place of a division: k_codes
-// 370 -> 114 us and k_quantize 422 -> 174 us for 4M points.
+// to [0, scale - 1]; scale is 2^21 or 2^30 and inv is scale / size, rounded. With
+// d = p - lo, rounded, as both take it, and t = scale d / size exact: the definition's
+// quotient is t within 2^-53 t (scale d is exact, one rounding), t' = d inv is t within
+// 2 * 2^-53 t, so for t up to 2^30 the two are within 3 * 2^-23 = 0.375 * 2^-20 of each
+// other. (d is at most hi - lo, so t passes 2^30 only by the rounding of a binary32 size;
+// both results are then scale - 1.) Added to 2^32, t' is rounded to a multiple of 2^-20,
+// off by at most 0.5 of them: 0.875 in all. So when the sum's fraction is none of 0 and
+// 2^20 - 1 of these steps, the whole part is the definition's. Otherwise, and for every t'
+// that is not in [0, 2^32), the definition decides. Three binary64 operations in place of a
+// division: k_codes 370 -> 114 us and k_quantize 422 -> 174 us for 4M points.
 __device__ __noinline__ uint32_t quantize_exact(double d, double size, double scale) {
     double t = 0.0;
     if (size > 0.0) t = floor(__ddiv_rn(__dmul_rn(scale, d), size));
@@ -438,7 +443,11 @@ cudaError_t encode_device(const float* xyz, const uint32_t* rgba, uint64_t n64, 
     if (e == cudaSuccess) e = cudaMemsetAsync(bounds, 0, sizeof(Bounds), st);
     if (e == cudaSuccess) e = cudaMemsetAsync(bounds->lo, 0xFF, sizeof bounds->lo, st);
     if (e != cudaSuccess) return e;
-    const uint32_t grid = (uint32_t)std::min<uint64_t>((n64 + kThreads - 1) / kThreads, 152 * 8);
+    int dev = 0, sms = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const uint32_t grid = (uint32_t)std::min<uint64_t>((n64 + kThreads - 1) / kThreads, (uint64_t)sms * kBlocksPerSm);
     k_bounds<<<grid, kThreads, 0, st>>>(d_xyz, n, bounds);
     if (keep_order) {
         k_identity<<<grid, kThreads, 0, st>>>(n, idx[0]);
