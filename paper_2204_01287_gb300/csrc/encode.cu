@@ -12,9 +12,11 @@
 //
 // Every binary64 operation is an explicit round-to-nearest intrinsic in the
 // host encoder's order, or certified to give its result (quantize). For 4M points
-// the kernels take 0.8 ms: the sort 0.5 (each pass reads and writes 12 bytes a point,
-// 41 of its 63 us in the scatter), k_quantize 0.17 (gathers of 12 bytes by index, nine
-// binary64 operations a point; GB300 has 2 binary64 FMAs per clock and SM), k_codes 0.11.
+// the kernels take 0.8 ms: the sort 0.5 (63 us a pass, 41 of them k_scatter, whose integer
+// pipe is 52 % busy), k_quantize 0.17 and k_codes 0.11, both at the binary64 rate (that
+// pipe 69 and 84 % busy; GB300 has 2 binary64 FMAs per clock and SM). From some ten million
+// points on k_quantize waits for its gathers of 12 bytes by index instead (50M points:
+// 3.2 ms, 363 bytes a point read from memory, the binary64 pipe 42 %).
 #include <algorithm>
 #include <cstdint>
 

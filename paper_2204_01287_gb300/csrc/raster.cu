@@ -43,8 +43,9 @@ __device__ __forceinline__ void raise_error(Scratch s, uint32_t code, uint32_t i
 // in the stream has ended (programmatic launch): its blocks are scheduled and its
 // code and parameters fetched while the other drains, and it waits here before
 // it touches memory that a kernel of the stream writes. One kernel, k_raster_fast,
-// may go on without waiting (take_list). A frame of a 10M-point cloud 32.1 -> 25.3 us, an LOD frame
-// 38.4 -> 29.5 us, a 100M-point fly-through 86.2 -> 79.3 us.
+// may go on without waiting (take_list). Frames back to back: a 10M-point cloud 32.1 ->
+// 25.3 us, an LOD frame 38.4 -> 29.5 us, a 100M-point fly-through 86.2 -> 79.3 us. A frame
+// alone gains little: its launches do not queue up, so there is nothing to start before.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void start_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -1017,10 +1018,8 @@ __device__ __forceinline__ uint32_t raster_words(const ViewConst& vc, const DecC
     return raster_quad<PARTIAL>(vc, x, y, z, g, valid);
 }
 
-// Points [p0, p1) of one batch for one view at precision K. The loop over
-// groups of 4 is warp-uniform; STREAM loads bypass L1 (single view), the
-// multi-view kernel keeps the words in cache for the next view.
-// One lane's group of 4 points at g: load, decode, raster.
+// One lane's group of 4 points at g: load, decode, raster. STREAM loads bypass L1
+// (single view), the multi-view kernel keeps the words in cache for the next view.
 template <int K, bool STREAM, bool PARTIAL>
 __device__ __forceinline__ uint32_t raster_group(const CloudView& c, const ViewConst& vc,
                                                  const DecConst& d, uint32_t g, uint32_t valid) {
@@ -1031,17 +1030,17 @@ __device__ __forceinline__ uint32_t raster_group(const CloudView& c, const ViewC
     return raster_words<K, PARTIAL>(vc, d, q1, q2, q3, g, valid);
 }
 
+// Bulk prefetch of [p, p + bytes) into L2 (16-byte aligned start and size).
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p), "r"(bytes) : "memory");
+}
+
 // Points [p0, p1) of one batch for one view at precision K, 128 points per
 // warp step. Steps that lie wholly inside the range (all of them but the last
 // for batches that start on a multiple of 128, as batches of 10,240 do) need
 // no bounds checks; the first step of an unaligned range and the last step
 // carry a validity mask. STREAM loads bypass L1 (single view), the multi-view
 // kernel keeps the words in cache for the next view.
-// Bulk prefetch of [p, p + bytes) into L2 (16-byte aligned start and size).
-__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(p), "r"(bytes) : "memory");
-}
-
 template <int K, bool STREAM>
 __device__ __forceinline__ uint32_t segment(const CloudView& c, const ViewConst& vc,
                                             const DecConst& d, uint32_t p0, uint32_t p1,
@@ -1247,7 +1246,7 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
 #pragma unroll
     for (int j = 0; j < 4; ++j) slow |= !pixel_bracket(fv, cxy[j], cw[j], bx[j], by[j]);
     if (slow) {
-        // a bracket did not settle: the definition for all four (rare)
+        // a bracket did not settle: the definition for all four (see project_pairs)
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             float cx, cy;
@@ -1287,9 +1286,10 @@ __device__ __forceinline__ uint32_t raster_decoded(const FastView& fv, const f2_
 // The one-view fast kernel packs two points instead of two rows: every operand is a
 // pair of points' values, so no half has to be copied to fill a pair, and the
 // view's coefficients come from the kernel's parameters as pairs (a, a). Every
-// operation and its order are those of the certified path above. On a view as dense
-// as the 2B-point frame 44.7 warp instructions per 32 points, about 47.5 before; the raster pass of the 2B-point overview 3.30 -> 3.19 ms, of the
-// 200M-point one 383 -> 370 us.
+// operation and its order are those of the certified path above. 50M points as dense
+// as the 2B-point frame take 50.7 warp instructions per 32 points at that frame's image
+// size and about 45 at 256x196, where fewer brackets stay open (about 47.5 before); the raster
+// pass of the 2B-point overview 3.30 -> 3.19 ms, of the 200M-point one 383 -> 370 us.
 
 // The view's coefficients, each twice.
 struct PairView {
@@ -1396,7 +1396,10 @@ __device__ __forceinline__ void project_pairs(const PairView& v, const PairPos& 
         py[2 * h + 1] = (uint32_t)(by >> 32);
     }
     if (!sure) {
-        // a bracket did not settle: the definition for all four (rare)
+        // A bracket did not settle: the definition for all four. A point is open with
+        // probability (W + H) 2^-20 at most, a warp step of 128 points with up to 5 % at
+        // 256x196, 31 % at 1920x1080 (25 % counted on the 2B-point overview), 40 % at
+        // 2016x2240, so on large images this is a part of the cost.
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const int s = (j & 1) * 32;
@@ -1580,9 +1583,9 @@ __device__ __forceinline__ void segment_fast_views(const CloudView& c, const Vie
 
 // Points [p0, p1) of a certified batch at precision K for views 0 and 1 of a
 // two-view launch (vmask: bit v set when view v is certified at K): one decode
-// per step as in segment_fast_views, two points per instruction, then each view with its constants read at
-// fixed parameter offsets, as in the one-view kernel (a view index that is
-// only known at run time makes them loads).
+// per step as in segment_fast_views, two points per instruction, then each view
+// with its constants read at fixed parameter offsets, as in the one-view kernel (a
+// view index that is only known at run time makes them loads).
 template <int K>
 __device__ __forceinline__ void segment_fast_pair(const CloudView& c, const ViewTable& vt,
                                                   const PairView& v0, const PairView& v1,
@@ -2640,10 +2643,13 @@ static cudaError_t launch_early(void (*kernel)(Params...), dim3 grid, unsigned t
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
     cfg.stream = st;
-    // Blocks that wait hold their SM's slots. Captured launches get plain edges,
-    // since graphs are what programs replay on several streams at once (16 views of
-    // 1M points on three streams: 80 us a frame with early starts, 66 us without; one
-    // view of 10M points on one stream: 28 and 30 us).
+    // Blocks that wait hold their SM's slots, which costs where several streams fill the
+    // chip and gains where a frame's kernels follow one another on one. Eager launches
+    // start early: one view of 10M points on one stream 36.5 -> 25.8 us, 16 views of 1M
+    // points 73.1 -> 67.4 us on one stream, 56.0 -> 57.5 us on three; the serving lanes, also
+    // several streams, are not told apart and lose 1 % (32 requests 800 -> 810 us).
+    // Captured ones have plain edges: replayed on three streams the 16 views took 80 us a
+    // frame with early starts, 66 us without.
     cfg.attrs = &early;
     cfg.numAttrs = capturing(st) ? 0 : 1;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
