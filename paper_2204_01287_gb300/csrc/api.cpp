@@ -398,25 +398,22 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
     pc_status rc = ensure_capacity(*slot, cl.n_entries, cl.is_lod ? cl.n_batches : 0);
     if (rc == PC_OK) rc = ensure_hqs(*slot, views, nviews, maxv);
     if (rc != PC_OK) return rc;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    cudaStreamIsCapturing(st, &cs);
+    const bool callers = capturing(st);   // the frame goes into a caller's graph
     const bool timing = timing_on.load();
-    const bool graph = (cfg.flags & PC_CFG_GRAPHS) && !timing &&
-                       cs == cudaStreamCaptureStatusNone && st != nullptr;
+    const bool graph = (cfg.flags & PC_CFG_GRAPHS) && !timing && !callers && st != nullptr;
     if (graph) {
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
     uint32_t kernels = 0;
-    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, graph || capturing(st), fo, &kernels);
+    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, graph || callers, fo, &kernels);
     launches += kernels;
     if (rc != PC_OK && !graph) {
         // The last pass, which leaves the scratch at zero, is missing: clear it behind
         // what was launched, for whatever uses it next (a replayed graph passes no
         // call of the library). While a caller captures, that part and its clearing
         // are the graph's and the scratch is as it was.
-        if (clear_scratch(*slot, false) != cudaSuccess && cs == cudaStreamCaptureStatusNone &&
-            slot->unclean == Unclean::kNo)
+        if (clear_scratch(*slot, false) != cudaSuccess && !callers && slot->unclean == Unclean::kNo)
             slot->unclean = Unclean::kFrame;
     }
     if (graph) {
