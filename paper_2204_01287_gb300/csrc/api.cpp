@@ -240,11 +240,11 @@ uint32_t Ctx::views_per_launch(const Cloud& cl) const {
 }
 
 // The kernels of one frame: per launch group, clear and cull / raster / shade /
-// resolve. *kernels: how many.
+// resolve. *kernels: how many; *branches: launch groups in two branches.
 pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                             const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
                             uint32_t maxv, bool timing, bool captured, const FrameOpts& fo,
-                            uint32_t* kernels) {
+                            uint32_t* kernels, uint32_t* branches) {
     CloudView cv = cl.view();
     if (fo.first || fo.count < cl.n_batches) {
         // a shard: the kernels see only the batches of the range (their point
@@ -319,7 +319,10 @@ pc_status Ctx::launch_frame(const Cloud& cl, const pc_view* views, uint32_t nvie
         Scratch s = slot->scratch;
         s.frame = 0;
         if (!captured) s.frame = slot->scratch.frame = next_frame(slot->scratch.frame);
-        e = launch_raster(cv, vt, s, shape, captured ? slot->second_branch() : nullptr, st, &raster_kernels);
+        const Branch* branch = nullptr;
+        if (captured && vt.n == 1 && may_certify(vt.v[0].flags)) branch = slot->second_branch();
+        e = launch_raster(cv, vt, s, shape, branch, st, &raster_kernels);
+        *branches += branch != nullptr;
         if (e != cudaSuccess) return cuda_fail(e, "raster launch");
         if (fe) cudaEventRecord(fe->ev[3], st);
         if (shade) {
@@ -405,8 +408,8 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         cudaError_t e = cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
     }
-    uint32_t kernels = 0;
-    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, graph || callers, fo, &kernels);
+    uint32_t kernels = 0, branches = 0;
+    rc = launch_frame(cl, views, nviews, fbs, st, slot, maxv, timing, graph || callers, fo, &kernels, &branches);
     launches += kernels;
     if (rc != PC_OK && !graph) {
         // The last pass, which leaves the scratch at zero, is missing: clear it behind
@@ -426,11 +429,13 @@ pc_status Ctx::render(const Cloud& cl, const pc_view* views, uint32_t nviews,
         if (e != cudaSuccess) return cuda_fail(e, "graph capture");
         // one instantiated graph per launch layout, so that programs which alternate
         // between layouts (plain and dilated views, with and without a colour pass) keep
-        // updating: the number of kernels tells the layouts of one view count apart
+        // updating: the numbers of kernels (at most 8 a group) and of branches tell the
+        // layouts of one view count apart
         uint64_t shaded = 0;
         for (uint32_t v = 0; v < nviews; ++v) shaded |= (uint64_t)(hqs_mode(views[v].flags) != 0);
         const uint64_t key = ((uint64_t)nviews << 8) | maxv | ((uint64_t)cl.is_lod << 40) |
-                             (shaded << 41) | ((uint64_t)fo.resolve_only << 42) | ((uint64_t)kernels << 43);
+                             (shaded << 41) | ((uint64_t)fo.resolve_only << 42) | ((uint64_t)kernels << 43) |
+                             ((uint64_t)branches << 55);
         cudaGraphExec_t& exec = slot->graphs[key];
         if (exec) {
             cudaGraphExecUpdateResultInfo info;

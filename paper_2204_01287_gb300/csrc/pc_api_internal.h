@@ -125,7 +125,8 @@ struct Ctx {
     void set_tune(Cloud& cl, uint32_t nviews, const Tune& t);
     pc_status launch_frame(const Cloud& cl, const pc_view* views, uint32_t nviews,
                            const pc_framebuffer* fbs, cudaStream_t st, Slot* slot, uint32_t maxv,
-                           bool timing, bool captured, const FrameOpts& fo, uint32_t* kernels);
+                           bool timing, bool captured, const FrameOpts& fo, uint32_t* kernels,
+                           uint32_t* branches);
     pc_status render(const Cloud& cl, const pc_view* views, uint32_t nviews,
                      const pc_framebuffer* fbs, cudaStream_t st, Slot* slot,
                      const FrameOpts& fo = FrameOpts());

@@ -159,7 +159,10 @@ cudaError_t launch_raster(const CloudView&, const ViewTable& vt, Scratch s, Rast
     // a captured launch has no number (every replay would repeat it), others one of their own
     if ((g_recording != nullptr) != (s.frame == 0) || (s.frame && s.frame <= g_last_frame)) ++g_misnumbered;
     if (s.frame) g_last_frame = s.frame;
-    if (branch) ++g_branches;
+    if (branch) {
+        ++g_branches;
+        run([] {});   // another topology
+    }
     if (fails("raster")) return cudaErrorLaunchFailure;
     *launched = vt.n == 1 ? 2 : 1;
     for (int i = 0; i < *launched; ++i) run([] {});
@@ -395,7 +398,8 @@ static void graphs_of_alternating_layouts() {
     World w(PC_CFG_GRAPHS);
     const std::vector<std::vector<uint32_t>> layouts = {
         {0u, 0u}, {0u, PC_VIEW_DILATE}, {PC_VIEW_DILATE, PC_VIEW_DILATE}, {PC_VIEW_HQS, 0u},
-        {PC_VIEW_HQS_PACKED, 0u}, {PC_VIEW_HQS_PACKED, PC_VIEW_DILATE}};
+        {PC_VIEW_HQS_PACKED, 0u}, {PC_VIEW_HQS_PACKED, PC_VIEW_DILATE},
+        {0u}, {PC_VIEW_FORCE_K(3)}, {PC_VIEW_NO_EARLY_DEPTH}, {PC_VIEW_FORCE_K(2) | PC_VIEW_DILATE}};
     for (const auto& l : layouts) CHECK(w.frame(l) == PC_OK);
     const int made = g_instantiated;
     CHECK(made <= (int)layouts.size());
@@ -420,7 +424,10 @@ static void captured_frames_branch() {
     g_last_frame = 0;
     World w(PC_CFG_GRAPHS);
     for (int i = 0; i < 3; ++i) CHECK(w.frame() == PC_OK && g_branches == 2 + i);
-    CHECK(g_misnumbered == 0 && g_instantiated == 3 && g_dirty == 0);
+    // views without a certified batch have nothing for the second branch
+    for (uint32_t f : {(uint32_t)PC_VIEW_FORCE_K(3), (uint32_t)PC_VIEW_NO_EARLY_DEPTH}) CHECK(w.frame({f}) == PC_OK);
+    CHECK(w.frame({0u, 0u}) == PC_OK && g_branches == 4);
+    CHECK(g_misnumbered == 0 && g_instantiated == 5 && g_dirty == 0);
 }
 
 static const std::map<std::string, void (*)()>& scenarios() {
